@@ -59,9 +59,10 @@ extern "C" {
 
 #define LETKF_FP32  0          /* plain FP32 CUDA-core analysis                                */
 #define LETKF_MIXED 1          /* split-precision: for 17 <= k <= 128 the localized Gram runs on
-                                  the tensor cores (tcgen05, FP16 hi+lo operands, FP32
-                                  accumulation; for k <= 32 two grid points share one
-                                  operand tile); for k <= 16 it stays on CUDA cores        */
+                                  the tensor cores on every grid (from 1,024 grid points on as
+                                  LETKF_GRAM_TENSOR below; on smaller ones with FP16 hi+lo
+                                  operands and FP32 accumulation; for k <= 32 two grid points
+                                  share one operand tile); for k <= 16 as in LETKF_FP32     */
 
 /* Eigensolve schedules (same results up to rounding; see letkf_config.eig_schedule). */
 #define LETKF_EIG_AUTO        0  /* the handle picks one: at its first analysis the schedules
@@ -104,18 +105,25 @@ extern "C" {
                                     against the observation error).  A probe's eigenvalues come
                                     from a tridiagonalization and an eigenvalue-only QL.      */
 
-/* FP32 Gram tile schedules for k >= 17 (letkf_config.gram_tile; k <= 16 has one schedule and
- * LETKF_MIXED uses the tensor cores for k >= 17, so the choice applies to LETKF_FP32 only). */
-#define LETKF_GRAM_AUTO   0  /* the handle times both on its first analysis' first chunk and
-                                keeps the faster; cached per problem shape for the process,
-                                so handles of the same shape run the same arithmetic        */
+/* FP32 Gram schedules (letkf_config.gram_tile; applies to LETKF_FP32 only, and PIPE / TEAM to
+ * k >= 17 only: k <= 16 has one CUDA-core schedule). */
+#define LETKF_GRAM_AUTO   0  /* LETKF_GRAM_TENSOR from 1,024 grid points on, where the network's
+                                products fit its buffer (n_obs x k (k + 3) / 2 entries of 6
+                                bytes within 2 GiB) and coordinates and cutoff are below 65536
+                                and 2896 cells.  Otherwise (k >= 17) the handle times PIPE and
+                                TEAM on its first analysis' first chunk and keeps the faster;
+                                cached per problem shape for the process, so handles of the
+                                same shape run the same arithmetic                          */
 #define LETKF_GRAM_PIPE   1  /* one CTA per SM over 7 x 2 points (k <= 64; 8 x 6 for k <= 32,
                                 3 x 1 for k <= 128), per-point compacted entries, operands
                                 double-buffered by cp.async                                */
 #define LETKF_GRAM_TEAM   2  /* two CTAs per SM over 4 x 2 points (k <= 64; 8 x 4, 2 x 1), the
                                 weights of a chunk in shared memory, a weight test per
                                 candidate in the multiply-add loop                         */
-#define LETKF_GRAM_TENSOR 3  /* (reported only) the tensor-core Gram of LETKF_MIXED          */
+#define LETKF_GRAM_TENSOR 3  /* (reported only) tensor cores: the Gram matrices of all grid points as
+                                one product over the observation points, three BF16 parts per
+                                operand (24 significant bits), FP32 sums; LETKF_MIXED's
+                                split-FP16 form on grids below 1,024 points                 */
 
 /* ---- problem statement --------------------------------------------------
  * Follows the paper's statement of the problem (Sec. II-B): the grid, the
@@ -165,7 +173,7 @@ typedef struct letkf_stats {
                                   cycle led by this handle): the kernel nodes of its
                                   captured graph; 0 before the first cycle               */
     int32_t gram_tile;         /* LETKF_GRAM_PIPE / TEAM / TENSOR in use; AUTO (0) until the
-                                  first analysis resolves it                             */
+                                  first analysis resolves it (between PIPE and TEAM)     */
 } letkf_stats;
 
 /* Device time of the phases of the most recent forecast and analysis (milliseconds, CUDA

@@ -29,6 +29,13 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr int64_t kDefaultChunkBytes = 1ll << 30;  // 1 GiB: 65,536 points at k = 64
+// The one-product Gram form (gram_gemm.cu): most bytes of its products (0.9 GB at 1024^2, k = 64,
+// every fourth point observed), and the smallest grid it takes: at 32 x 32 points it measured
+// 1.03 to 3.6 times as fast as the better CUDA-core schedule (16 to 37 us against 18 to 133, k = 8
+// to 128, r = 3 to 12), at 128 x 128 1.9 to 9.2 times; below 1,024 points (four tiles of work at
+// most per pair tile) the CUDA-core schedules stay.
+constexpr int64_t kGemmMaxBytes = 2ll << 30;
+constexpr int kGemmMinPoints = 1024;
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -42,6 +49,8 @@ struct Plan {
     int nmem = 0, V = 0, LV = 0, kp = 0;
     int tile_w = 1, tile_h = 1;
     bool tensor_gram = false;  // mixed precision with k in 17..128: tcgen05 split-FP16 Gram
+    bool gemm = false;         // the Gram matrices as one tensor-core product (gram_gemm.cu)
+    int np = 0;                // its pairs, padded
     int eig_schedule = LETKF_EIG_FUSED;  // as configured; AUTO keeps both schedules' scratch
     int rcap = 0;              // split schedule: rotation record entries per point
     int chunk_rows = 0;
@@ -52,7 +61,7 @@ struct Plan {
     float inv_c = 0.0f;  // Gaspari-Cohn: 1 / (sqrt(10/3) r)
     // byte offsets inside the workspace
     size_t off_state[2], off_force, off_xg, off_obs_xy, off_cell_start, off_cell_obs, off_rinv,
-        off_yf, off_yb, off_ybar, off_yo, off_orec, off_gram, off_cvec, off_nloc, off_nloc_all,
+        off_yf, off_yb, off_ybar, off_yo, off_orec, off_z, off_oxy, off_pairs, off_offs, off_gram, off_cvec, off_nloc, off_nloc_all,
         off_eigval, off_de, off_taus, off_rot, off_nrot, off_list, off_pre_list, off_status,
         total;
 };
@@ -125,6 +134,16 @@ int make_plan(const letkf_config *c, Plan *p) {
         p->inv2r2 = (float)(1.0 / (2.0 * r * r));
         p->inv_c = (float)(1.0 / (sqrt(10.0 / 3.0) * r));
     }
+    // The Gram matrices as one product over the observation points (gram_gemm.cu): squared
+    // distances exact in FP32, coordinates in 16 bits, and the products of all observation
+    // points within kGemmMaxBytes.
+    p->np = lk::gram_gemm_pairs(c->k);
+    const int64_t zbytes = (int64_t)c->n_obs * p->np * 3 * 2;
+    p->gemm = c->n_obs > 0 && c->nx < 65536 && c->ny < 65536 &&
+              (c->loc_kind == LETKF_LOC_NONE || p->d2max < (1 << 23)) && zbytes <= kGemmMaxBytes &&
+              (p->tensor_gram || c->gram_tile == LETKF_GRAM_AUTO) &&
+              p->npts >= (size_t)kGemmMinPoints;
+    if (p->gemm) p->tile_h = std::lcm(p->tile_h, lk::kGemmTile);
     // bins: smallest power-of-two edge (>= 8) whose patch of one Gram tile fits the kernel
     const int maxc = lk::gram_max_cells();
     for (p->cs = 8;; p->cs *= 2) {
@@ -170,6 +189,10 @@ int make_plan(const letkf_config *c, Plan *p) {
     p->off_ybar = take((size_t)p->LV * sizeof(float));
     p->off_yo = take((size_t)p->LV * sizeof(float));
     p->off_orec = take(p->tensor_gram ? (size_t)p->LV * sizeof(float4) : 0);
+    p->off_z = take(p->gemm ? (size_t)zbytes : 0);
+    p->off_oxy = take(p->gemm ? (size_t)c->n_obs * sizeof(float2) : 0);
+    p->off_pairs = take(p->gemm ? (size_t)p->np * sizeof(int) : 0);
+    p->off_offs = take(p->gemm ? (size_t)p->np * sizeof(int) : 0);
     p->off_gram = take(p->chunk_pts * c->k * c->k * sizeof(float));
     p->off_cvec = take(p->chunk_pts * c->k * sizeof(float));
     p->off_nloc = take(p->chunk_pts * sizeof(int));
@@ -222,6 +245,11 @@ struct letkf_handle {
     float *xg = nullptr, *rinv = nullptr, *yf = nullptr, *yb = nullptr, *ybar = nullptr,
           *yo = nullptr, *gram = nullptr, *cvec = nullptr, *eigval = nullptr;
     float4 *orec = nullptr;
+    bool gemm = false;            // the one-product Gram form is in use
+    __nv_bfloat16 *z = nullptr;   // its products, observation points, pair tables, tensor map
+    float2 *oxy = nullptr;
+    int *pairs = nullptr, *offs = nullptr;
+    lk::TmaMap zmap;
     int2 *obs_xy = nullptr;
     int *cell_start = nullptr, *cell_obs = nullptr, *nloc = nullptr, *nloc_all = nullptr,
         *status = nullptr;
@@ -350,6 +378,8 @@ int enqueue_forecast(letkf_handle *h, int nsteps) {
     return mark(h, 1);
 }
 
+constexpr int kGemmFlag = 24;   // word of the status block: a product of gram_z is not finite
+
 int enqueue_obs(letkf_handle *h) {
     const Plan &p = h->plan;
     lk::ObsOpArgs o;
@@ -365,6 +395,7 @@ int enqueue_obs(letkf_handle *h) {
     o.yf = h->yf;
     o.yb = h->yb;
     o.ybar = h->ybar;
+    if (h->gemm) o.clear = h->status + kGemmFlag;
     CK(lk::launch_obs_operator(o, h->stream));
     return LETKF_OK;
 }
@@ -395,6 +426,25 @@ lk::GramArgs gram_args(letkf_handle *h, int y0, int y1) {
 // Gram matrices and c of the chunk of rows [y0, y1) (the chunk index selects the records pass)
 int enqueue_gram_chunk(letkf_handle *h, int chunk, int y0, int y1) {
     const lk::GramArgs g = gram_args(h, y0, y1);
+    if (h->gemm) {
+        lk::GemmArgs m;
+        m.net = h->net;
+        m.nx = h->cfg.nx;
+        m.ny = h->cfg.ny;
+        m.k = h->cfg.k;
+        m.y_begin = y0;
+        m.y_end = y1;
+        m.oxy = h->oxy;
+        m.offs = h->offs;
+        m.z = h->z;
+        m.np = h->plan.np;
+        m.gram = h->gram;
+        m.cvec = h->cvec;
+        m.flag = h->status + kGemmFlag;
+        if (chunk == 0) CK(lk::launch_gram_z(m, g, h->pairs, h->stream));
+        CK(lk::launch_gram_gemm(m, h->zmap, h->status, h->tc_ctas, h->stream));
+        return LETKF_OK;
+    }
     if (h->plan.tensor_gram && chunk == 0) CK(lk::launch_obs_records(g, h->orec, h->stream));
     if (h->plan.tensor_gram)
         CK(lk::launch_gram_tc(g, h->status, h->tc_ctas, h->stream));
@@ -403,8 +453,14 @@ int enqueue_gram_chunk(letkf_handle *h, int chunk, int y0, int y1) {
     return LETKF_OK;
 }
 
+// Local observation points of the chunk's grid points (the one-product Gram form takes the
+// static counts, the others count while they gather).
+const int *chunk_nloc(const letkf_handle *h, int y0) {
+    return h->gemm ? h->nloc_all + (size_t)y0 * h->cfg.nx : h->nloc;
+}
+
 // The handle's status block (kAlign bytes, zeroed at letkf_init): word 0 the latched status
-// bits, words 16..18 the grouped launches' work counters, bytes 128..151 the Chebyshev
+// bits, words 16..18 the grouped launches' work counters, word 24 the one-product Gram form's flag, bytes 128..151 the Chebyshev
 // transform's cumulative counts (points, products, points handed on).
 unsigned long long *work_counters(letkf_handle *h) {
     return reinterpret_cast<unsigned long long *>(h->status + 32);
@@ -418,7 +474,7 @@ lk::EigArgs eig_args(letkf_handle *h, int y0, int y1) {
     e.sqrt_infl = (float)sqrt((double)h->cfg.infl);
     e.gram = h->gram;
     e.cvec = h->cvec;
-    e.nloc = h->nloc;
+    e.nloc = chunk_nloc(h, y0);
     e.x = h->xg;
     e.pt0 = (long long)y0 * h->cfg.nx;
     e.npts = (y1 - y0) * h->cfg.nx;
@@ -648,7 +704,7 @@ int enqueue_analysis(letkf_handle *h, letkf_probe *probe) {
                 const long long lp = probe->points[i] - pt0;
                 if (lp < 0 || lp >= npts) continue;
                 if (probe->nloc)
-                    CK(cudaMemcpyAsync(probe->nloc + i, h->nloc + lp, sizeof(int),
+                    CK(cudaMemcpyAsync(probe->nloc + i, chunk_nloc(h, y0) + lp, sizeof(int),
                                        cudaMemcpyDeviceToHost, h->stream));
                 if (probe->gram)
                     CK(cudaMemcpyAsync(probe->gram + (size_t)i * k * k, h->gram + lp * k * k,
@@ -949,6 +1005,12 @@ int letkf_init(const letkf_config *cfg, void *workspace, size_t workspace_bytes,
     h->ybar = (float *)(w + plan.off_ybar);
     h->yo = (float *)(w + plan.off_yo);
     h->orec = plan.tensor_gram ? (float4 *)(w + plan.off_orec) : nullptr;
+    if (plan.gemm) {
+        h->z = (__nv_bfloat16 *)(w + plan.off_z);
+        h->oxy = (float2 *)(w + plan.off_oxy);
+        h->pairs = (int *)(w + plan.off_pairs);
+        h->offs = (int *)(w + plan.off_offs);
+    }
     h->gram = (float *)(w + plan.off_gram);
     h->cvec = (float *)(w + plan.off_cvec);
     h->nloc = (int *)(w + plan.off_nloc);
@@ -1031,9 +1093,23 @@ int letkf_init(const letkf_config *cfg, void *workspace, size_t workspace_bytes,
         (cheb_candidate(plan.eig_schedule, cfg->k) &&
          lk::eigen_cheb_prepare(cfg->k, &h->cheb_grid) != cudaSuccess))
         return fail(LETKF_ECUDA);
-    if (plan.tensor_gram) {
+    if (plan.gemm) {
+        std::vector<float2> oxy(L);
+        for (int j = 0; j < L; ++j)
+            oxy[j] = make_float2((float)xy[cobs[j]].x, (float)xy[cobs[j]].y);
+        std::vector<int> pairs(plan.np), offs(plan.np);
+        lk::gram_gemm_tables(cfg->k, pairs.data(), offs.data());
+        int ok = 0;
+        if (cudaMemcpy(h->oxy, oxy.data(), L * sizeof(float2), cudaMemcpyHostToDevice) ||
+            cudaMemcpy(h->pairs, pairs.data(), plan.np * sizeof(int), cudaMemcpyHostToDevice) ||
+            cudaMemcpy(h->offs, offs.data(), plan.np * sizeof(int), cudaMemcpyHostToDevice) ||
+            lk::gram_gemm_prepare(h->z, L, plan.np, &h->zmap, &ok) != cudaSuccess)
+            return fail(LETKF_ECUDA);
+        h->gemm = ok != 0;   // without the driver's tensor-map encoder the other forms serve
+    }
+    if (plan.tensor_gram || plan.gemm) {
         int sms = 0;
-        if (lk::gram_tc_prepare(plan.kp) != cudaSuccess ||
+        if ((plan.tensor_gram && lk::gram_tc_prepare(plan.kp) != cudaSuccess) ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess)
             return fail(LETKF_ECUDA);
         h->tc_ctas = sms;  // one CTA per SM: each holds all 512 tensor-memory columns
@@ -1069,7 +1145,7 @@ int letkf_init(const letkf_config *cfg, void *workspace, size_t workspace_bytes,
         plan.eig_schedule == LETKF_EIG_AUTO ? cached_eig_schedule(h) : plan.eig_schedule;
     h->stats.eig_schedule = h->eig_schedule;
     // the Gram: tensor cores (mixed), the one team schedule (k <= 16), else as configured
-    if (plan.tensor_gram)
+    if (plan.tensor_gram || h->gemm)
         h->gram_tile = LETKF_GRAM_TENSOR;
     else if (plan.kp <= 16)
         h->gram_tile = LETKF_GRAM_TEAM;

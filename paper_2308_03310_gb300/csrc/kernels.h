@@ -1,6 +1,7 @@
 // Host-side launchers of the library's kernels (internal to libletkf).
 #pragma once
 
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -71,6 +72,7 @@ struct ObsOpArgs {
     float *yf;              // [nmem][L*V] h(x_m)
     float *yb;              // [L*V][kp]  h(x_m) - mean, zero in columns k..kp-1
     float *ybar;            // [L*V]      mean minus the variable's reference (1 for rho)
+    int *clear = nullptr;   // a device word set to zero (optional)
 };
 cudaError_t launch_obs_operator(const ObsOpArgs &a, cudaStream_t s);
 cudaError_t launch_count_local(const ObsNet &net, int nx, int ny, int *nloc, cudaStream_t s);
@@ -109,6 +111,30 @@ cudaError_t launch_gram(const GramArgs &a, cudaStream_t s);
 int gram_tile_width(int kp, int team);
 int gram_tile_height(int kp, int team);
 int gram_max_cells();
+
+// ---- gram_gemm.cu -------------------------------------------------------------
+// The Gram matrices as one (grid points x observation points) x (observation points x pairs)
+// product on the tensor cores, three BF16 parts per operand.
+constexpr int kGemmTile = 16;        // edge of a tile of grid points
+constexpr int kGemmC = 1 << 30;      // offs[m] >= kGemmC: entry offs[m] - kGemmC of c
+struct GemmArgs {
+    ObsNet net;
+    int nx, ny, k;
+    int y_begin, y_end;     // grid rows of this chunk
+    const float2 *oxy;      // [L] observation points in bin order
+    const int *offs;        // [np] a pair's offset in the k x k slot, or in c, or -1 (padding)
+    __nv_bfloat16 *z;       // [3][L][np] the pairs' products, three parts, rows in bin order
+    int np;                 // pairs, padded (gram_gemm_pairs)
+    float *gram, *cvec;     // as in GramArgs
+    int *flag;              // raised by launch_gram_z where some product is not finite
+};
+int gram_gemm_pairs(int k);
+void gram_gemm_tables(int k, int *pairs, int *offs);   // [gram_gemm_pairs(k)] each
+// the tensor map of z; *ok = 0 where the driver offers no encoder
+cudaError_t gram_gemm_prepare(const void *z, int L, int np, TmaMap *map, int *ok);
+cudaError_t launch_gram_z(const GemmArgs &a, const GramArgs &g, const int *pairs, cudaStream_t s);
+cudaError_t launch_gram_gemm(const GemmArgs &a, const TmaMap &map, int *status, int max_ctas,
+                             cudaStream_t s);
 
 // ---- eigen.cu -----------------------------------------------------------------
 struct EigArgs {

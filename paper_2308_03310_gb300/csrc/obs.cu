@@ -19,6 +19,7 @@ __global__ void __launch_bounds__(128) obs_operator_kernel(ObsOpArgs a) {
     const size_t npts = (size_t)a.nx * a.ny;
     const int V = __popc(a.obs_vars & 7);
     const int LV = a.L * V;
+    if (a.clear && blockIdx.x == 0 && threadIdx.x == 0) *a.clear = 0;
     for (int l = warp; l < a.L; l += nwarps) {
         const int2 o = a.xy[l];
         const size_t p = (size_t)o.y * a.nx + o.x;
