@@ -893,6 +893,55 @@ int enqueue_group(letkf_handle *const *hs, int n, int nsteps) {
     return LETKF_OK;
 }
 
+// A group cycle from its captured graph, captured first where there is none yet (inside a
+// GroupScope).
+int replay_group(letkf_handle *const *hs, int n, int nsteps) {
+    letkf_handle *h = hs[0];
+    // the captured graph of this membership, schedules, state buffers and step count
+    std::vector<unsigned long long> ids(n);
+    std::vector<int> cur(n), sched(n);
+    for (int i = 0; i < n; ++i) {
+        ids[i] = hs[i]->serial;
+        cur[i] = hs[i]->cur;
+        sched[i] = hs[i]->eig_schedule;
+    }
+    letkf_handle::GroupGraph *gg = nullptr;
+    for (auto &e : h->group_graphs)
+        if (e.members == ids && e.cur == cur && e.sched == sched && e.nsteps == nsteps)
+            gg = &e;
+    if (!gg) {
+        if (h->group_graphs.size() >= 8) {  // bounded cache: drop the oldest
+            if (h->group_graphs.front().exec) cudaGraphExecDestroy(h->group_graphs.front().exec);
+            h->group_graphs.erase(h->group_graphs.begin());
+        }
+        CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeRelaxed));
+        const int rc = enqueue_group(hs, n, nsteps);
+        cudaGraph_t g = nullptr;
+        const cudaError_t ec = cudaStreamEndCapture(h->stream, &g);
+        for (int i = 0; i < n; ++i) hs[i]->cur = cur[i];
+        if (rc) {
+            if (g) cudaGraphDestroy(g);
+            return rc;
+        }
+        if (ec != cudaSuccess) return cuda_fail(h, ec);
+        letkf_handle::GroupGraph e;
+        e.members = ids;
+        e.cur = cur;
+        e.sched = sched;
+        e.nsteps = nsteps;
+        e.kernels = graph_kernel_nodes(g);
+        const cudaError_t ei = cudaGraphInstantiate(&e.exec, g, 0);
+        cudaGraphDestroy(g);
+        if (ei != cudaSuccess) return cuda_fail(h, ei);
+        h->group_graphs.push_back(e);
+        gg = &h->group_graphs.back();
+    }
+    CK(cudaGraphLaunch(gg->exec, h->stream));
+    h->stats.cycle_kernels = gg->kernels;
+    for (int i = 0; i < n; ++i) hs[i]->cur ^= (forecast_flips(nsteps) & 1);
+    return LETKF_OK;
+}
+
 int status_to_code(int bits) {
     if (bits & lk::ST_NONFINITE) return LETKF_ENONFINITE;
     if (bits & lk::ST_NOTCONV) return LETKF_ENOTCONV;
@@ -1459,51 +1508,11 @@ int letkf_group_cycle(letkf_handle *const *hs, int32_t n, int32_t nsteps, const 
         if (pending) {
             if ((rc = enqueue_group(hs, n, nsteps))) return rc;
             h->stats.cycle_kernels = 0;
-            return group_fence(hs, n, true);
+        } else if ((rc = replay_group(hs, n, nsteps))) {
+            return rc;
         }
-        // the captured graph of this membership, schedules, state buffers and step count
-        std::vector<unsigned long long> ids(n);
-        std::vector<int> cur(n), sched(n);
-        for (int i = 0; i < n; ++i) {
-            ids[i] = hs[i]->serial;
-            cur[i] = hs[i]->cur;
-            sched[i] = hs[i]->eig_schedule;
-        }
-        letkf_handle::GroupGraph *gg = nullptr;
-        for (auto &e : h->group_graphs)
-            if (e.members == ids && e.cur == cur && e.sched == sched && e.nsteps == nsteps)
-                gg = &e;
-        if (!gg) {
-            if (h->group_graphs.size() >= 8) {  // bounded cache: drop the oldest
-                if (h->group_graphs.front().exec) cudaGraphExecDestroy(h->group_graphs.front().exec);
-                h->group_graphs.erase(h->group_graphs.begin());
-            }
-            CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeRelaxed));
-            rc = enqueue_group(hs, n, nsteps);
-            cudaGraph_t g = nullptr;
-            const cudaError_t ec = cudaStreamEndCapture(h->stream, &g);
-            for (int i = 0; i < n; ++i) hs[i]->cur = cur[i];
-            if (rc) {
-                if (g) cudaGraphDestroy(g);
-                return rc;
-            }
-            if (ec != cudaSuccess) return cuda_fail(h, ec);
-            letkf_handle::GroupGraph e;
-            e.members = ids;
-            e.cur = cur;
-            e.sched = sched;
-            e.nsteps = nsteps;
-            e.kernels = graph_kernel_nodes(g);
-            const cudaError_t ei = cudaGraphInstantiate(&e.exec, g, 0);
-            cudaGraphDestroy(g);
-            if (ei != cudaSuccess) return cuda_fail(h, ei);
-            h->group_graphs.push_back(e);
-            gg = &h->group_graphs.back();
-        }
-        CK(cudaGraphLaunch(gg->exec, h->stream));
-        h->stats.cycle_kernels = gg->kernels;
-        for (int i = 0; i < n; ++i) hs[i]->cur ^= (forecast_flips(nsteps) & 1);
     }
+    // (outside the scope: the handles have their own streams again, which the fence orders)
     return group_fence(hs, n, true);
 }
 
