@@ -38,11 +38,12 @@ METRIC = "LETKF grid-pt analyses/s + p99 cycle latency, mixed vs FP32 at stated 
 UNIT = "grid-pt analyses/s"
 FLUSH_BYTES = 256 << 20
 FP32_LANES_PER_SM = 128
+LBM_STEPS_PER_LAUNCH = 4
 SMS = 152
 
 # Algorithmic work per unit:
 #   lbm_step      72 B per node and member per launch (one FP32 read and one write of the nine
-#                 populations; two time steps per launch) + 8 B per node of force
+#                 populations; four time steps per launch) + 8 B per node of force
 #   transpose     2 x 36 k B per grid point (read + write of the 9 x k block)
 #   obs_operator  36 B per (observation point, member) read + 4 V B per (point, member) written x2
 #   gram          k (k + 1) flops per local observed scalar per grid point (the upper triangle
@@ -247,16 +248,16 @@ def cheb_flops(k, counts):
 
 
 def kernel_work(w, k, npts, mean_local_obs, V, nobs_pts, chunks, steps, schedule=1,
-                cheb_counts=None):
+                cheb_counts=None, steps_per_launch=2):
     """Algorithmic work of one cycle per kernel: (unit, amount, launches).  For the CHEBYSHEV
     schedule the eigen phase's work follows the device counters of the cycle (cheb_counts);
     without them it falls back to the RATIONAL count."""
     eig = (cheb_flops(k, cheb_counts) if schedule == 5 and cheb_counts
            else eigen_flops_per_point(k, schedule) * npts)
     return {
-        # two steps per launch: one read and one write of the state (+ the force) per launch
-        "lbm_step": ("GB", (72.0 * npts * k + 8.0 * npts) * (steps // 2 + steps % 2) / 1e9,
-                     steps // 2 + steps % 2),
+        # one read and one write of the state (+ the force) per launch of steps_per_launch steps
+        "lbm_step": ("GB", (72.0 * npts * k + 8.0 * npts) * -(-steps // steps_per_launch) / 1e9,
+                     -(-steps // steps_per_launch)),
         "obs_operator": ("GB", (36.0 + 8.0 * V) * nobs_pts * k / 1e9, 1),
         "transpose_in": ("GB", 72.0 * k * npts / 1e9, 1),
         "gram": ("TFLOP", (k * (k + 1) + 2 * k) * V * mean_local_obs * npts / 1e12, chunks),
@@ -273,16 +274,17 @@ def lbm_rates(w, forecast_ms, peaks):
     updates = float(w.n_points) * w.k * w.steps_per_cycle
     mlups = updates / (forecast_ms * 1e-3) / 1e6
     eq_gbs = (72.0 * updates + 8.0 * w.n_points * w.steps_per_cycle) / (forecast_ms * 1e-3) / 1e9
-    return {"mlups": mlups, "mlups_per_member": mlups / w.k, "steps_per_launch": 2,
+    return {"mlups": mlups, "mlups_per_member": mlups / w.k,
+            "steps_per_launch": LBM_STEPS_PER_LAUNCH,
             "single_step_equivalent_gbs": eq_gbs,
             "single_step_equivalent_frac": eq_gbs / peaks["hbm_gbs"]}
 
 
 def roofline_table(work, ms, peaks, sm_mhz, tensor_gram=False):
-    """Per kernel: achieved = algorithmic work / device time against its peak.  The mixed
-    form's Gram runs on the tensor cores (FP16 operands: the measured sustained BF16 GEMM
-    rate, FP16 and BF16 have the same nominal dense rate); its split form executes 2 tensor
-    flops per algorithmic flop ([Xl; Xh] Xh^T), so frac <= 0.5 even at the tensor peak."""
+    """Per kernel: achieved = algorithmic work / device time against its peak.  A Gram on the
+    tensor cores is set against the measured sustained BF16 GEMM rate (FP16 and BF16 have the
+    same nominal dense rate); the algorithmic count is the per-scalar one (k (k + 1) + 2 k per
+    local observed scalar), not what the one-product form executes."""
     out = {}
     total = sum(ms.values())
     for name, (unit, amount, launches) in work.items():
@@ -1505,8 +1507,8 @@ def measure(w, members, setup, yos, device, precision, steps, warm, world, eig_s
         peaks["fp32_tflops"] = peak32["tflops"]
     sm_mhz = peaks["sm_max_mhz"] or 2070.0
     work = kernel_work(w, w.k, w.n_points, st.mean_local_obs, exp.V, exp.L, st.n_chunks,
-                       w.steps_per_cycle, exp.stats().eig_schedule, cheb)
-    tensor_gram = precision == L.LETKF_MIXED and 17 <= w.k <= 128
+                       w.steps_per_cycle, exp.stats().eig_schedule, cheb, LBM_STEPS_PER_LAUNCH)
+    tensor_gram = exp.stats().gram_tile == L.LETKF_GRAM_TENSOR
     table = roofline_table(work, ms, peaks, sm_mhz, tensor_gram)
     top = max(table, key=lambda n: table[n]["ms_per_cycle"])
     t = table[top]

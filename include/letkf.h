@@ -180,7 +180,7 @@ typedef struct letkf_stats {
  * events on the handle's stream), the breakdown of Fig. 3 of the paper for one GPU. */
 typedef struct letkf_timings {
     float   forecast_ms;       /* all D2Q9 steps of the last forecast                   */
-    int32_t forecast_steps;    /* steps (= kernel launches) in it                       */
+    int32_t forecast_steps;    /* steps in it (up to four per kernel launch)            */
     float   obs_ms;            /* observation operator                                   */
     float   transpose_in_ms;   /* member-major -> grid-point-major                       */
     float   gram_ms;           /* localized Gram + innovation projection, all chunks     */

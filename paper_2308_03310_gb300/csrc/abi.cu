@@ -241,7 +241,7 @@ struct letkf_handle {
     float *state[2] = {nullptr, nullptr};
     int cur = 0;
     float2 *force = nullptr;
-    lk::LbmTma lbm_tma;           // TMA descriptors of the two-step D2Q9 staging
+    int lbm_rows[lk::kLbmSteps] = {1, 1, 1, 1};   // rows per segment of the D2Q9 launches
     float *xg = nullptr, *rinv = nullptr, *yf = nullptr, *yb = nullptr, *ybar = nullptr,
           *yo = nullptr, *gram = nullptr, *cvec = nullptr, *eigval = nullptr;
     float4 *orec = nullptr;
@@ -356,22 +356,17 @@ int mark(letkf_handle *h, int idx) {
     return LETKF_OK;
 }
 
-// Ping-pong buffer flips of a forecast: two steps per launch, a single step for an odd rest.
-int forecast_flips(int nsteps) { return nsteps / 2 + (nsteps & 1); }
+// Ping-pong buffer flips of a forecast: one per launch of up to kLbmSteps steps.
+int forecast_flips(int nsteps) { return nsteps / lk::kLbmSteps + (nsteps % lk::kLbmSteps != 0); }
 
 int enqueue_forecast(letkf_handle *h, int nsteps) {
     const Plan &p = h->plan;
     int rc = mark(h, 0);
     if (rc) return rc;
-    for (int s = 0; s + 2 <= nsteps; s += 2) {
-        CK(lk::launch_lbm_2step(h->state[h->cur], h->state[h->cur ^ 1], h->force, h->cfg.nx,
-                                h->cfg.ny, p.nmem, h->cfg.tau, h->stream, &h->lbm_tma,
-                                h->status));
-        h->cur ^= 1;
-    }
-    if (nsteps & 1) {
-        CK(lk::launch_lbm_step(h->state[h->cur], h->state[h->cur ^ 1], h->force, h->cfg.nx,
-                               h->cfg.ny, p.nmem, h->cfg.tau, h->stream));
+    for (int left = nsteps; left > 0; left -= lk::kLbmSteps) {
+        CK(lk::launch_lbm(h->state[h->cur], h->state[h->cur ^ 1], h->force, h->cfg.nx, h->cfg.ny,
+                          p.nmem, h->cfg.tau, std::min(left, lk::kLbmSteps), h->lbm_rows,
+                          h->stream));
         h->cur ^= 1;
     }
     if (h->timing) h->fc_steps = nsteps;
@@ -1130,10 +1125,13 @@ int letkf_init(const letkf_config *cfg, void *workspace, size_t workspace_bytes,
     h->net.loc_gc = cfg->loc_kind == LETKF_LOC_GC;
     h->net.inv_c = plan.inv_c;
 
-    if (lk::lbm_prepare() != cudaSuccess ||
-        lk::lbm_tma_build(h->state[0], h->state[1], h->force, cfg->nx, cfg->ny, plan.nmem,
-                          &h->lbm_tma) != cudaSuccess ||
-        lk::gram_prepare(plan.kp) != cudaSuccess ||
+    {
+        int sms = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess)
+            return fail(LETKF_ECUDA);
+        lk::lbm_plan(cfg->nx, cfg->ny, plan.nmem, sms, h->lbm_rows);
+    }
+    if (lk::gram_prepare(plan.kp) != cudaSuccess ||
         lk::eigen_prepare(cfg->k, &h->eig_blocks) != cudaSuccess ||
         (plan.eig_schedule != LETKF_EIG_FUSED &&
          lk::eigen_split_prepare(cfg->k, &h->eig_split) != cudaSuccess) ||

@@ -1,32 +1,34 @@
 // Batched ensemble D2Q9 lattice Boltzmann kernels (Sec. II-A).
 //
-// One time step of Eq. 1 for every member at once: each thread reads the nine
-// populations of one node of one member, forms the moments (Eqs. 2-3), applies
-// the BGK relaxation towards the second-order D2Q9 equilibrium plus the body-force
-// source F_q = 3 w_q c_q . F, and pushes each post-collision population to the
-// neighbour x + c_q (periodic).  The stored state is the post-streaming f.
+// Time steps of Eq. 1 for every member at once: the nine populations of a node give the moments
+// (Eqs. 2-3), the BGK relaxation towards the second-order D2Q9 equilibrium plus the body-force
+// source F_q = 3 w_q c_q . F, and every post-collision population moves to the neighbour
+// x + c_q (periodic).  The stored state is the post-streaming f.
 //
 // Layout: member-major structure of arrays g[m][q][y][x] (the paper's LBM layout
 // X[m, N_v, N_x], Sec. IV-A), FP32, holding the deviation g_q = f_q - w_q from the
-// rest state (exact weights).  Every load and store is a coalesced 4-byte access of a warp along x;
-// one step moves 72 bytes per lattice update and is HBM bound.
+// rest state (exact weights).
 //
-// Two steps per launch (temporal blocking): a CTA stages a TX x TY tile of one member with a
-// periodic halo of two nodes in shared memory (rows copied in 16-byte runs), collides every staged node and pushes into a
-// second tile (halo one), collides again and pushes the second step's populations of the
-// tile's own nodes to HBM.  Per two steps a node is read ~1.3 times (the halos) and written
-// once: ~84 bytes instead of 144.  The collision runs on pairs of neighbouring nodes with
-// packed FP32 arithmetic; it is the same function in both kernels, so the arithmetic is the
-// same as two single steps.
+// Up to four steps per launch (lbm_kernel<T>), in registers.  A warp owns a window of 64 columns of
+// one member, two neighbouring ones per lane, and marches along y: per row it loads the nine
+// populations (coalesced, one row ahead), and the T steps run as a pipeline of T stages, stage s
+// one row behind stage s - 1.  A collision's outputs stream to the stage after it: along x with
+// one shuffle per direction and pair, along y by waiting in registers (those with c_y = -1 are
+// used at once, c_y = 0 one row later, c_y = +1 two rows later).  The last stage's populations are
+// streamed the same way and stored, coalesced.  A window loses one column per side and step, so
+// neighbouring windows overlap by the halo, and so do the segments of rows a member is cut into.
+// No shared memory and no barrier: a form that kept four steps' rows in shared memory (36
+// accesses of 8 bytes per pair of nodes and step, four barriers per eight rows) was bound by
+// them, at 1.26 to 1.45 ms per four steps of 1024^2, k = 64, whatever the tile.
 //
-// Staging: where the window lies inside the grid (the tile is not at a periodic edge) and nx is
-// a multiple of 4, one thread loads it with two bulk tensor copies (TMA: the nine population
-// planes of the member as one 3-D box, the force as one 2-D box of interleaved components),
-// their completion counted in bytes on an mbarrier; elsewhere every thread issues 16-byte (or
-// 4-byte) cp.async copies with the periodic wrap.  Both put the same values in the same places.
-#include <cuda.h>   // CUtensorMap and the tensor-map encoder's types
-
-#include <mutex>
+// Measured (four steps, with a force; before: two launches of two steps through shared memory
+// with the collision written as g + omega (g_eq - g) per direction):
+//   1024^2, k = 64: 1759 -> 1031 us (64 % of the copy rate in its own 4.8 GB);
+//   256^2, k = 32: 71.1 -> 42.1 us; 509 x 380, k = 20: 185 -> 74.5 us; 64^2, k = 20: 8.6 -> 8.3 us.
+// Bound: the FP32 pipe (53 % active at 256^2, k = 64) behind the latency of three warps per
+// scheduler, which is what 168 registers allow; 128 registers (four warps) spill and measured
+// 1337 us, the row loop without its unrolling by two (moves between the waiting rows) 1148 us.
+#include <math.h>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -57,137 +59,89 @@ __device__ __forceinline__ float2 rcp2(float2 x) {
     return fma2(y, e, y);
 }
 
-// c_q . v for a lattice direction known at compile time (no multiplications by 0 or +-1).
-template <int CX, int CY>
-__device__ __forceinline__ float2 cdot2(float2 vx, float2 vy) {
-    if constexpr (CX == 0) return CY > 0 ? vy : neg2(vy);
-    else if constexpr (CY == 0) return CX > 0 ? vx : neg2(vx);
-    else return add2(CX > 0 ? vx : neg2(vx), CY > 0 ? vy : neg2(vy));
-}
-
-// Direction Q (0..3) and its opposite 8 - Q: the equilibrium of the pair from its symmetric
-// and antisymmetric parts, w (a +- b) with a = base + 4.5 rho (c.u)^2 and b = 3 rho c.u, then
-// the BGK relaxation and the force term +- 3 w c.F.
-template <bool kForce, int Q>
-__device__ __forceinline__ void collide_pair(const float2 (&g)[NV], float2 ux, float2 uy,
-                                             float2 base, float2 r3, float2 r45, float2 f3x,
-                                             float2 f3y, float2 omega, float2 (&out)[NV]) {
-    const float2 w = dup2(wq(Q));
-    const float2 cu = cdot2<cx(Q), cy(Q)>(ux, uy);
-    const float2 a = fma2(mul2(r45, cu), cu, base);
-    const float2 b = mul2(r3, cu);
-    const float2 gp = mul2(w, add2(a, b)), gm = mul2(w, sub2(a, b));  // equilibria of Q, 8 - Q
-    float2 sp = fma2(omega, sub2(gp, g[Q]), g[Q]);
-    float2 sm = fma2(omega, sub2(gm, g[8 - Q]), g[8 - Q]);
-    if (kForce) {
-        const float2 fq = mul2(w, cdot2<cx(Q), cy(Q)>(f3x, f3y));
-        sp = add2(sp, fq);
-        sm = sub2(sm, fq);
-    }
-    out[Q] = sp;
-    out[8 - Q] = sm;
+// The collision's constants, from omega = 1 / tau in FP32 (host, FP64).  They satisfy
+// rest + 9 rho = 1 and rest + 12 mom = 1 (rho, mom as two FP32 words each) and quad = 3 quad6
+// exactly, so that a collision conserves mass and momentum up to the rounding of its sums: a
+// constant off by one ulp would act on every node and step with the same sign (an error of
+// 6e-6 after 100 steps, measured, against 5e-7).
+struct LbmCoef {
+    float rest;             // 1 - omega
+    float rho, rho_lo;      // omega / 9
+    float mom, mom_lo;      // omega / 12
+    float nquad6, quad, quad8, quad4;   // -omega / 6, omega / 2, omega / 8, omega / 4
+};
+LbmCoef lbm_coef(float tau) {
+    LbmCoef c;
+    const double omega = (double)(1.0f / tau);
+    c.rest = (float)(1.0 - omega);
+    const double t = 1.0 - (double)c.rest;   // the relaxation in effect (omega for tau <= 2)
+    c.rho = (float)(t / 9.0);
+    c.rho_lo = (float)(t / 9.0 - (double)c.rho);
+    c.mom = (float)(t / 12.0);
+    c.mom_lo = (float)(t / 12.0 - (double)c.mom);
+    int e = 0;
+    const double m = frexp(t / 6.0, &e);     // 22 significant bits: 3 quad6 is an FP32 number
+    const double q6 = ldexp(rint(ldexp(m, 22)), e - 22);
+    c.nquad6 = (float)-q6;
+    c.quad = (float)(3.0 * q6);
+    c.quad8 = 0.25f * c.quad;
+    c.quad4 = 0.5f * c.quad;
+    return c;
 }
 
 // BGK collision with the body-force source for two nodes: post-collision populations out[q]
-// from the nodes' deviations g[q] (Eq. 1, Sec. II-A).  f^eq_q = w_q (rho + rho (3 c.u +
-// 4.5 (c.u)^2 - 1.5 |u|^2)) written for the deviations: geq_q = w_q (drho - 1.5 rho |u|^2 +
-// 4.5 rho (c.u)^2 + 3 rho c.u), evaluated per pair of opposite directions (q, 8 - q), whose
-// terms differ only in the sign of c.u.
+// from the nodes' deviations g[q] (Eq. 1, Sec. II-A).
+//
+// out = (1 - omega) g + omega g_eq + 3 w c.F, with the directions paired (q, 8 - q): the
+// equilibrium's even part is w (drho + 4.5 (c.j)(c.u) - 1.5 j.u) and its odd part 3 w c.j (j = rho u),
+// so no density multiplies the momentum again.  With P = j_x u_x, Q = j_y u_y, R = j_x u_y,
+//   even (times omega): rest 4 b, x axis b + omega P / 2, y axis b + omega Q / 2, diagonals
+//     b / 4 + omega (P + Q) / 8 +- omega R / 4, b = omega (drho / 9 - (P + Q) / 6);
+//   odd: 4 m_x, 4 m_y, m_x +- m_y, m = (omega j + F) / 12.
+// 61 packed operations for two nodes (the form g + omega (g_eq - g) per direction took 95).  Error
+// after 100 steps against 64 bits (tau = 0.52, u = 0.02, emulated): 2.1e-6 -> 5e-7.
 template <bool kForce>
 __device__ __forceinline__ void collide2(const float2 (&g)[NV], float2 fx, float2 fy,
-                                         float2 omega, float2 (&out)[NV]) {
-    const float2 g01 = add2(g[0], g[1]);
-    const float2 drho = add2(add2(add2(g01, add2(g[2], g[3])), add2(add2(g[4], g[5]),
-                                                                  add2(g[6], g[7]))), g[8]);
-    const float2 jx = sub2(add2(add2(g[2], g[5]), g[8]), add2(add2(g[0], g[3]), g[6]));
-    const float2 jy = sub2(add2(add2(g[6], g[7]), g[8]), add2(g01, g[2]));
-    const float2 rho = add2(dup2(1.0f), drho);
-    const float2 rinv = rcp2(rho);
+                                         const LbmCoef &c, float2 (&out)[NV]) {
+    const float2 s0 = add2(g[0], g[8]), s1 = add2(g[1], g[7]), s2 = add2(g[2], g[6]),
+                 s3 = add2(g[3], g[5]);
+    const float2 d0 = sub2(g[8], g[0]), d1 = sub2(g[7], g[1]), d2 = sub2(g[6], g[2]),
+                 d3 = sub2(g[5], g[3]);
+    const float2 drho = add2(add2(add2(s0, s2), add2(s1, s3)), g[4]);
+    const float2 jx = add2(sub2(d0, d2), d3), jy = add2(add2(d0, d2), d1);
+    const float2 rinv = rcp2(add2(dup2(1.0f), drho));
     const float2 ux = mul2(jx, rinv), uy = mul2(jy, rinv);
-    const float2 base = fma2(mul2(dup2(-1.5f), rho), fma2(ux, ux, mul2(uy, uy)), drho);
-    const float2 r3 = mul2(dup2(3.0f), rho), r45 = mul2(dup2(4.5f), rho);
-    const float2 f3x = mul2(dup2(3.0f), fx), f3y = mul2(dup2(3.0f), fy);
-    collide_pair<kForce, 0>(g, ux, uy, base, r3, r45, f3x, f3y, omega, out);
-    collide_pair<kForce, 1>(g, ux, uy, base, r3, r45, f3x, f3y, omega, out);
-    collide_pair<kForce, 2>(g, ux, uy, base, r3, r45, f3x, f3y, omega, out);
-    collide_pair<kForce, 3>(g, ux, uy, base, r3, r45, f3x, f3y, omega, out);
-    out[4] = fma2(omega, sub2(mul2(dup2(wq(4)), base), g[4]), g[4]);
-}
-
-template <bool kForce>
-__global__ void __launch_bounds__(256) lbm_step_kernel(const float *__restrict__ gin,
-                                                       float *__restrict__ gout,
-                                                       const float2 *__restrict__ force,
-                                                       int nx, int ny, float omega) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= nx || y >= ny) return;
-    const size_t npts = (size_t)nx * ny;
-    const size_t mbase = (size_t)blockIdx.z * NV * npts;
-    const size_t p = (size_t)y * nx + x;
-
-    float2 g[NV], out[NV];
-#pragma unroll
-    for (int q = 0; q < NV; ++q) g[q] = dup2(__ldcs(gin + mbase + q * npts + p));
-    float2 fx = dup2(0.0f), fy = dup2(0.0f);
+    const float2 P = mul2(jx, ux), Q = mul2(jy, uy), R = mul2(jx, uy), PQ = add2(P, Q);
+    const float2 b =
+        fma2(dup2(c.rho), drho, fma2(dup2(c.nquad6), PQ, mul2(dup2(c.rho_lo), drho)));
+    const float2 ax = fma2(dup2(c.quad), P, b), ay = fma2(dup2(c.quad), Q, b);
+    const float2 e = fma2(dup2(0.25f), b, mul2(dup2(c.quad8), PQ)), h = mul2(dup2(c.quad4), R);
+    const float2 ap = add2(e, h), am = sub2(e, h);
+    float2 lx = mul2(dup2(c.mom_lo), jx), ly = mul2(dup2(c.mom_lo), jy);
     if (kForce) {
-        const float2 F = __ldg(force + p);
-        fx = dup2(F.x);
-        fy = dup2(F.y);
+        lx = fma2(dup2(1.0f / 12.0f), fx, lx);
+        ly = fma2(dup2(1.0f / 12.0f), fy, ly);
     }
-    collide2<kForce>(g, fx, fy, dup2(omega), out);
-    const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
-    const int ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
-    float *dst = gout + mbase;
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-        const int xd = cx(q) < 0 ? xm : (cx(q) > 0 ? xp : x);
-        const int yd = cy(q) < 0 ? ym : (cy(q) > 0 ? yp : y);
-        __stcs(dst + q * npts + (size_t)yd * nx + xd, out[q].x);
-    }
+    const float2 mx = fma2(dup2(c.mom), jx, lx), my = fma2(dup2(c.mom), jy, ly);
+    const float2 mp = add2(mx, my), mm = sub2(mx, my);
+    const float2 r = dup2(c.rest);
+    out[4] = fma2(dup2(4.0f), b, mul2(r, g[4]));
+    out[8] = add2(fma2(r, g[8], ap), mp);
+    out[0] = sub2(fma2(r, g[0], ap), mp);
+    out[2] = add2(fma2(r, g[2], am), mm);
+    out[6] = sub2(fma2(r, g[6], am), mm);
+    out[7] = fma2(dup2(4.0f), my, fma2(r, g[7], ay));
+    out[1] = fma2(dup2(-4.0f), my, fma2(r, g[1], ay));
+    out[5] = fma2(dup2(4.0f), mx, fma2(r, g[5], ax));
+    out[3] = fma2(dup2(-4.0f), mx, fma2(r, g[3], ax));
 }
 
-// Two-step tile: 64 x 12 output nodes, 256 threads, four CTAs (51 KB of shared memory each)
-// per SM.  Measured against 64 x 8/16/20, 32 x 16 and 128 x 8 tiles and 128/512-thread CTAs:
-// the fastest at 256^2 (k = 32) and 1024^2 (k = 64).
-constexpr int kTX = 64;                  // output tile width
-constexpr int kTY = 12;                  // output tile height
-constexpr int kStep2Threads = 256;
-constexpr int kStep2MinBlocks = 4;
-
-template <int TX, int TY>
-constexpr size_t step2_smem() {          // staged tile (halo 2, x window widened to 16 bytes)
-    return (size_t)(TX + 8) * (TY + 4) * (NV + 2) * sizeof(float);   // and its force
-}
-
-static_assert(sizeof(TmaMap) == sizeof(CUtensorMap) && alignof(TmaMap) >= 64, "tensor map image");
-
-constexpr unsigned long long kTmaWaitNs = 2000000000ull;   // bound of a staging wait (2 s)
-
-__device__ __forceinline__ unsigned long long lbm_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-__device__ __forceinline__ bool tma_bar_try(uint32_t bar) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(bar)
-        : "memory");
-    return done != 0;
-}
-// bounded wait for the staging barrier's first phase
-__device__ __forceinline__ bool tma_bar_wait(uint32_t bar) {
-    if (tma_bar_try(bar)) return true;
-    const unsigned long long t0 = lbm_ns();
-    for (;;) {
-        if (tma_bar_try(bar)) return true;
-        if (lbm_ns() - t0 > kTmaWaitNs) return false;
-    }
-}
+constexpr int kWin = 64;                      // columns of a warp's window
+constexpr int kLbmWarps = 4;                  // warps (windows) per CTA
+constexpr int kLbmBlocks = 3;                 // CTAs per SM
+// halo columns on either side of a strip: T, rounded up to whole pairs
+constexpr int lbm_halo(int T) { return (T + 1) & ~1; }
+constexpr int lbm_strip(int T) { return kWin - 2 * lbm_halo(T); }
 
 // Periodic wrap of a coordinate at most one period outside [0, n).
 __device__ __forceinline__ int wrap1(int a, int n) {
@@ -195,206 +149,163 @@ __device__ __forceinline__ int wrap1(int a, int n) {
     return (unsigned)r < (unsigned)n ? r : posmod(a, n);   // grids narrower than the halo
 }
 
-__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)
-                     __cvta_generic_to_shared(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)
-                     __cvta_generic_to_shared(dst)), "l"(src) : "memory");
+// Streamed populations whose consumers' rows are still to come: c_y = 0 of the last row, c_y = +1
+// of the last and of the one before.
+struct Waiting {
+    float2 zero[3], up1[3], up2[3];
+};
+
+// A collision's outputs displaced by c_x: lane c holds columns 2c, 2c + 1.
+__device__ __forceinline__ void stream_x(const float2 (&o)[NV], float2 (&s)[NV]) {
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        if (cx(q) == 0) s[q] = o[q];
+        else if (cx(q) > 0) s[q] = make_float2(__shfl_up_sync(0xffffffffu, o[q].y, 1), o[q].x);
+        else s[q] = make_float2(o[q].y, __shfl_down_sync(0xffffffffu, o[q].x, 1));
+    }
 }
 
-template <bool kForce, int TX, int TY, int NT, int MINB>
-__global__ void __launch_bounds__(NT, MINB) lbm_2step_kernel(const float *__restrict__ gin,
-                                                             float *__restrict__ gout,
-                                                             const float2 *__restrict__ force,
-                                                             int nx, int ny, float omega_s,
-                                                             const __grid_constant__ TmaMap tg,
-                                                             const __grid_constant__ TmaMap tf,
-                                                             int use_tma, int *status) {
-    // staged step-t window: x in [x0 - 4, x0 + TX + 4), y in [y0 - 2, y0 + TY + 2); the nodes
-    // two beyond the tile on each side are the halo, the outer two columns only align the
-    // window's rows to 16 bytes
-    constexpr int AX = TX + 8, AY = TY + 4;
-    constexpr int BX = TX + 2, BY = TY + 2;      // step-(t+1) nodes, origin (x0 - 1, y0 - 1)
-    constexpr int HX = TX + 4;                   // collided columns 2 .. AX - 3
-    static_assert(TX % 4 == 0 && HX % 2 == 0 && BX % 2 == 0, "16-byte rows, node pairs");
-    extern __shared__ __align__(128) float sm[];
-    __shared__ __align__(8) uint64_t tbar;
-    float *A = sm;                                               // [q][AY][AX]
-    float2 *Fs = reinterpret_cast<float2 *>(sm + NV * AX * AY);  // force over A's nodes
-    static_assert((NV * AX * AY * 4) % 128 == 0, "the force box starts 128-byte aligned");
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+// The populations that reach the row above the one just streamed (s), and the wait of the rest.
+__device__ __forceinline__ void stream_y(const float2 (&s)[NV], Waiting &w, float2 (&g)[NV]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        g[k] = s[k];                // c_y = -1
+        g[3 + k] = w.zero[k];
+        g[6 + k] = w.up2[k];
+        w.up2[k] = w.up1[k];
+        w.up1[k] = s[6 + k];
+        w.zero[k] = s[3 + k];
+    }
+}
+
+// T steps.  Unit u: strip (fastest), segment of H rows, member.  kEven: nx is even, so a window's
+// pairs are 8-byte aligned and never split by the periodic wrap.
+template <int T, bool kForce, bool kEven>
+__global__ void __launch_bounds__(32 * kLbmWarps, kLbmBlocks)
+    lbm_kernel(const float *__restrict__ gin, float *__restrict__ gout,
+               const float2 *__restrict__ force, int nx, int ny, int H, int strips, int segs,
+               long long units, LbmCoef coef) {
+    constexpr int HX = lbm_halo(T), TX = lbm_strip(T);
+    const long long u = (long long)blockIdx.x * kLbmWarps + (threadIdx.x >> 5);
+    if (u >= units) return;
+    const int c = threadIdx.x & 31;
+    const int strip = (int)(u % strips), seg = (int)(u / strips % segs);
     const size_t npts = (size_t)nx * ny;
-    const size_t mbase = (size_t)blockIdx.z * NV * npts;
-    const int tid = threadIdx.x;
-    const float2 omega = dup2(omega_s);
-    // ---- stage the window: a window inside the grid by TMA (the maps exist only where nx is a
-    // multiple of 4, so x0 - 4 is a 16-byte boundary); otherwise with cp.async, every copy of
-    // the thread in flight before the one wait: runs of four nodes (16 bytes) where nx is a
-    // multiple of 4 -- x0 is, so every run starts on a 16-byte boundary, also where it wraps --
-    // single nodes otherwise
-    const bool by_tma = use_tma && x0 >= 4 && x0 + TX + 4 <= nx && y0 >= 2 && y0 + TY + 2 <= ny;
-    if (by_tma) {
-        const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&tbar);
-        if (tid == 0) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
-            asm volatile("fence.mbarrier_init.release.cluster;");
-        }
-        __syncthreads();
-        if (tid == 0) {
-            constexpr uint32_t bytes = NV * AX * AY * 4 + (kForce ? AX * AY * 8 : 0);
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
-                         "r"(bytes)
-                         : "memory");
-            asm volatile(
-                "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-                " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"((uint32_t)__cvta_generic_to_shared(A)),
-                "l"(reinterpret_cast<uint64_t>(&tg)), "r"(x0 - 4), "r"(y0 - 2),
-                "r"((int)blockIdx.z * NV), "r"(bar)
-                : "memory");
-            if (kForce)
-                asm volatile(
-                    "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::"
-                    "bytes [%0], [%1, {%2, %3}], [%4];" ::"r"((uint32_t)__cvta_generic_to_shared(Fs)),
-                    "l"(reinterpret_cast<uint64_t>(&tf)), "r"(2 * (x0 - 4)), "r"(y0 - 2), "r"(bar)
-                    : "memory");
-        }
-        // the outcome made uniform over the CTA; a timeout is never expected: report it, give
-        // the copies a second bounded wait to land, leave
-        if (__syncthreads_and(tma_bar_wait(bar)) == 0) {
-            if (tid == 0 && status) atomicOr(status, ST_TIMEOUT);
-            tma_bar_wait(bar);
-            return;
-        }
-    } else if ((nx & 3) == 0) {
-        constexpr int GX = AX / 4;
-        for (int e = tid; e < AY * GX; e += NT) {
-            const int ay = e / GX, gx = e - ay * GX;
-            const size_t p = (size_t)wrap1(y0 - 2 + ay, ny) * nx + wrap1(x0 - 4 + 4 * gx, nx);
-            float *a = A + ay * AX + 4 * gx;
-#pragma unroll
-            for (int q = 0; q < NV; ++q) cp_async16(a + q * AY * AX, gin + mbase + q * npts + p);
-            if (kForce) {
-                cp_async16(Fs + ay * AX + 4 * gx, force + p);
-                cp_async16(Fs + ay * AX + 4 * gx + 2, force + p + 2);
-            }
-        }
-    } else {
-        for (int e = tid; e < AX * AY; e += NT) {
-            const int ay = e / AX, ax = e - ay * AX;
-            const size_t p = (size_t)wrap1(y0 - 2 + ay, ny) * nx + wrap1(x0 - 4 + ax, nx);
-#pragma unroll
-            for (int q = 0; q < NV; ++q) cp_async4(A + (q * AY + ay) * AX + ax, gin + mbase + q * npts + p);
-            if (kForce) {
-                const float *F = reinterpret_cast<const float *>(force + p);
-                cp_async4(reinterpret_cast<float *>(Fs + e), F);
-                cp_async4(reinterpret_cast<float *>(Fs + e) + 1, F + 1);
-            }
-        }
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();
-    // ---- collision t of the tile and its halo, in place (a node owns its nine slots), two
-    // neighbouring nodes (ax, ax + 1), ax even, per thread
-    for (int e = tid; e < HX * AY / 2; e += NT) {
-        const int ay = (2 * e) / HX, ax = 2 + 2 * e - ay * HX;
-        const int i = ay * AX + ax;
-        float2 g[NV], out[NV];
-#pragma unroll
-        for (int q = 0; q < NV; ++q) g[q] = *reinterpret_cast<const float2 *>(A + q * AY * AX + i);
-        float2 fx = dup2(0.0f), fy = dup2(0.0f);
-        if (kForce) {
-            const float4 F = *reinterpret_cast<const float4 *>(Fs + i);
-            fx = make_float2(F.x, F.z);
-            fy = make_float2(F.y, F.w);
-        }
-        collide2<kForce>(g, fx, fy, omega, out);
-#pragma unroll
-        for (int q = 0; q < NV; ++q) *reinterpret_cast<float2 *>(A + q * AY * AX + i) = out[q];
-    }
-    __syncthreads();
-    // ---- streaming t -> t+1 as a pull from the collided neighbours, collision t+1, and the
-    // push of t+1 -> t+2 into the tile's own nodes in HBM; node pairs (bx, bx + 1), bx even
-    float *dst = gout + mbase;
-    for (int e = tid; e < BX * BY / 2; e += NT) {
-        const int by = (2 * e) / BX, bx = 2 * e - by * BX;
-        const int ay = by + 1, ax = bx + 3;                     // the first node's slot in A
-        float2 g[NV], out[NV];
+    const size_t mbase = (size_t)(u / strips / segs) * NV * npts;
+    const int x0 = strip * TX, ys = seg * H, ye = min(ys + H, ny);
+    const int xa = wrap1(x0 - HX + 2 * c, nx), xb = wrap1(x0 - HX + 2 * c + 1, nx);
+    const float *const src = gin + mbase;
+    // row l of the segment is y = ys - T + l (periodic), l < rows
+    const int rows = ye - ys + 2 * T;
+    int y = posmod(ys - T, ny);              // of the row to be loaded next
+    auto load = [&](float2 (&g)[NV], float2 &f0, float2 &f1) {
+        const size_t p = (size_t)y * nx;
 #pragma unroll
         for (int q = 0; q < NV; ++q) {
-            const float *src = A + (q * AY + ay - cy(q)) * AX + ax - cx(q);
-            // the pair's sources are 8-byte aligned where ax - c_x is even (c_x = +-1)
-            g[q] = cx(q) != 0 ? *reinterpret_cast<const float2 *>(src)
-                              : make_float2(src[0], src[1]);
+            const float *a = src + (size_t)q * npts + p;
+            g[q] = kEven ? __ldcs(reinterpret_cast<const float2 *>(a + xa))
+                         : make_float2(__ldcs(a + xa), __ldcs(a + xb));
         }
-        float2 fx = dup2(0.0f), fy = dup2(0.0f);
         if (kForce) {
-            const float2 F0 = Fs[ay * AX + ax], F1 = Fs[ay * AX + ax + 1];
-            fx = make_float2(F0.x, F1.x);
-            fy = make_float2(F0.y, F1.y);
+            if (kEven) {                     // the pair's force: one 16-byte load
+                const float4 f = __ldg(reinterpret_cast<const float4 *>(force + p + xa));
+                f0 = make_float2(f.x, f.y);
+                f1 = make_float2(f.z, f.w);
+            } else {
+                f0 = __ldg(force + p + xa);
+                f1 = __ldg(force + p + xb);
+            }
         }
-        collide2<kForce>(g, fx, fy, omega, out);
-        // targets (bx - 1 + h + c_x, by - 1 + c_y) of node h: inside the tile and the grid
-        const int tx0 = bx - 1, ty0 = by - 1;
-        bool vx[4], vy[3];
+        y = y + 1 == ny ? 0 : y + 1;
+    };
+    // targets: columns x0 + t, x0 + t + 1 of the strip and grid (for an even nx both or neither)
+    const int t = 2 * c - HX;
+    const bool in0 = t >= 0 && t < TX && x0 + t < nx, in1 = in0 && x0 + t + 1 < nx;
+    float *const dst = gout + mbase + (x0 + t);
+
+    Waiting w[T > 1 ? T - 1 : 1];
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-            vx[c] = (unsigned)(tx0 + c - 1) < (unsigned)TX && x0 + tx0 + c - 1 < nx;
+    for (int i = 0; i < (T > 1 ? T - 1 : 1); ++i)
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
-            vy[c] = (unsigned)(ty0 + c - 1) < (unsigned)TY && y0 + ty0 + c - 1 < ny;
-        const long long at = (long long)(y0 + ty0) * nx + (x0 + tx0);
-        // a pair's targets are 8-byte aligned where c_x = +-1 and nx is even (x0 + bx even):
-        // one float2 store where both are inside
-        const bool pair_ok = (nx & 1) == 0;
+        for (int k = 0; k < 3; ++k) w[i].zero[k] = w[i].up1[k] = w[i].up2[k] = make_float2(0.0f, 0.0f);
+    float2 fx[T], fy[T];                     // the force of the stages' rows
+#pragma unroll
+    for (int i = 0; i < T; ++i) fx[i] = fy[i] = make_float2(0.0f, 0.0f);
+    float2 nxt[NV], nf0 = fx[0], nf1 = fx[0];
+    load(nxt, nf0, nf1);
+#pragma unroll 2
+    for (int l = 0; l < rows; ++l) {
+        float2 g[NV], o[NV], s[NV];
+#pragma unroll
+        for (int q = 0; q < NV; ++q) g[q] = nxt[q];
+#pragma unroll
+        for (int i = T - 1; i > 0; --i) {
+            fx[i] = fx[i - 1];
+            fy[i] = fy[i - 1];
+        }
+        fx[0] = make_float2(nf0.x, nf1.x);
+        fy[0] = make_float2(nf0.y, nf1.y);
+        if (l + 1 < rows) load(nxt, nf0, nf1);
+#pragma unroll
+        for (int i = 0; i < T; ++i) {        // stage i + 1, row l - i
+            collide2<kForce>(g, fx[i], fy[i], coef, o);
+            stream_x(o, s);
+            if (i + 1 < T) stream_y(s, w[i], g);
+        }
+        // the last stage's row l - T + 1, pushed along y
+        const int yr = ys - T + l - (T - 1);
+        if (l < 2 * T - 2 || !in0) continue;
 #pragma unroll
         for (int q = 0; q < NV; ++q) {
-            float *d = dst + at + (long long)q * (long long)npts + cy(q) * nx + cx(q);
-            if (vy[cy(q) + 1]) {
-                const bool v0 = vx[cx(q) + 1], v1 = vx[cx(q) + 2];
-                if (cx(q) != 0 && pair_ok && v0 && v1) {
-                    __stcs(reinterpret_cast<float2 *>(d), out[q]);
-                } else {
-                    if (v0) __stcs(d, out[q].x);
-                    if (v1) __stcs(d + 1, out[q].y);
-                }
+            if (yr + cy(q) < ys || yr + cy(q) >= ye) continue;
+            float *d = dst + ((size_t)q * npts + (size_t)(yr + cy(q)) * nx);
+            if (kEven) {
+                __stcs(reinterpret_cast<float2 *>(d), s[q]);
+            } else {
+                __stcs(d, s[q].x);
+                if (in1) __stcs(d + 1, s[q].y);
             }
         }
     }
 }
 
-template <int TX, int TY, int NT, int MINB>
-cudaError_t set_step2_smem() {
-    cudaError_t e = cudaFuncSetAttribute(lbm_2step_kernel<true, TX, TY, NT, MINB>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)step2_smem<TX, TY>());
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(lbm_2step_kernel<false, TX, TY, NT, MINB>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)step2_smem<TX, TY>());
+// Rows per segment: the least estimated time.  A row of a segment (its 2 T halo rows and about two
+// for the first load included) takes a scheduler with one, two or three warps 1.7, 2.4 or 3 units
+// (a lone warp waits for its own chain of collisions); three warps fit.
+template <int T>
+int segment_rows(int nx, int ny, int nmem, int sms) {
+    const long long lines = (long long)((nx + lbm_strip(T) - 1) / lbm_strip(T)) * nmem;
+    constexpr int wmax = kLbmBlocks * kLbmWarps / 4;
+    static_assert(wmax == 3, "the units of a row");
+    const double unit[wmax] = {0.0, 1.7, 2.4};
+    int best = ny;
+    double least = 0.0;
+    for (int n = 1; n <= ny; ++n) {          // segments
+        const int H = (ny + n - 1) / n;
+        const long long w = (lines * ((ny + H - 1) / H) + 4 * sms - 1) / (4 * sms);
+        const double cost = ((double)(w / wmax * wmax) + unit[w % wmax]) * (H + 2 * T + 2);
+        if (n == 1 || cost < least) {
+            least = cost;
+            best = H;
+        }
+        if (H < 2) break;
+    }
+    return best;
 }
 
-template <int TX, int TY, int NT, int MINB>
-cudaError_t launch_2step(const float *gin, float *gout, const float2 *force, int nx, int ny,
-                         int nmem, float tau, cudaStream_t s, const LbmTma *tma, int *status) {
-    dim3 grid((nx + TX - 1) / TX, (ny + TY - 1) / TY, nmem);
-    const float omega = 1.0f / tau;
-    const size_t smem = step2_smem<TX, TY>();
-    // the state map of the buffer read, and the force map where the force is staged
-    const int b = !tma || !(tma->ok & 1) ? -1 : gin == tma->gptr[0] ? 0 : gin == tma->gptr[1] ? 1 : -1;
-    const int use = b >= 0 && (!force || (tma->ok & 2));
-    static const TmaMap none = {};
-    const TmaMap &tg = use ? tma->g[b] : none;
-    const TmaMap &tf = use && force ? tma->f : none;
-    if (force)
-        lbm_2step_kernel<true, TX, TY, NT, MINB><<<grid, NT, smem, s>>>(gin, gout, force, nx,
-                                                                        ny, omega, tg, tf, use,
-                                                                        status);
+template <int T, bool kForce>
+cudaError_t launch_steps(const float *gin, float *gout, const float2 *force, int nx, int ny,
+                         int nmem, float tau, cudaStream_t s, int rows) {
+    const int strips = (nx + lbm_strip(T) - 1) / lbm_strip(T), segs = (ny + rows - 1) / rows;
+    const long long units = (long long)strips * segs * nmem;
+    const unsigned grid = (unsigned)((units + kLbmWarps - 1) / kLbmWarps);
+    const LbmCoef coef = lbm_coef(tau);
+    if (nx % 2 == 0)
+        lbm_kernel<T, kForce, true><<<grid, 32 * kLbmWarps, 0, s>>>(gin, gout, force, nx, ny, rows,
+                                                                    strips, segs, units, coef);
     else
-        lbm_2step_kernel<false, TX, TY, NT, MINB><<<grid, NT, smem, s>>>(gin, gout, force, nx,
-                                                                         ny, omega, tg, tf, use,
-                                                                         status);
+        lbm_kernel<T, kForce, false><<<grid, 32 * kLbmWarps, 0, s>>>(gin, gout, force, nx, ny, rows,
+                                                                     strips, segs, units, coef);
     return cudaGetLastError();
 }
 
@@ -428,88 +339,28 @@ __global__ void macro_kernel(const float *__restrict__ rho, const float *__restr
 
 }  // namespace
 
-cudaError_t launch_lbm_step(const float *gin, float *gout, const float2 *force, int nx, int ny,
-                            int nmem, float tau, cudaStream_t s) {
+void lbm_plan(int nx, int ny, int nmem, int sms, int rows[kLbmSteps]) {
+    rows[0] = segment_rows<1>(nx, ny, nmem, sms);
+    rows[1] = segment_rows<2>(nx, ny, nmem, sms);
+    rows[2] = segment_rows<3>(nx, ny, nmem, sms);
+    rows[3] = segment_rows<4>(nx, ny, nmem, sms);
+}
+
+cudaError_t launch_lbm(const float *gin, float *gout, const float2 *force, int nx, int ny, int nmem,
+                       float tau, int steps, const int rows[kLbmSteps], cudaStream_t s) {
     if (nmem <= 0) return cudaSuccess;
-    const int bx = nx >= 128 ? 128 : ((nx + 31) / 32) * 32;
-    const int by = 256 / bx;
-    dim3 block(bx, by);
-    dim3 grid((nx + bx - 1) / bx, (ny + by - 1) / by, nmem);
-    const float omega = 1.0f / tau;
-    if (force)
-        lbm_step_kernel<true><<<grid, block, 0, s>>>(gin, gout, force, nx, ny, omega);
-    else
-        lbm_step_kernel<false><<<grid, block, 0, s>>>(gin, gout, force, nx, ny, omega);
-    return cudaGetLastError();
-}
-
-cudaError_t lbm_prepare() { return set_step2_smem<kTX, kTY, kStep2Threads, kStep2MinBlocks>(); }
-
-cudaError_t launch_lbm_2step(const float *gin, float *gout, const float2 *force, int nx, int ny,
-                             int nmem, float tau, cudaStream_t s, const LbmTma *tma, int *status) {
-    if (nmem <= 0) return cudaSuccess;
-    return launch_2step<kTX, kTY, kStep2Threads, kStep2MinBlocks>(gin, gout, force, nx, ny, nmem,
-                                                                   tau, s, tma, status);
-}
-
-namespace {
-using EncodeTiled = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
-                                 const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
-                                 const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                 CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-// the driver's tensor-map encoder, through the runtime (no link against the driver library)
-EncodeTiled encode_tiled() {
-    static EncodeTiled fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000,
-                                             cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiled>(p);
-    });
-    return fn;
-}
-}  // namespace
-
-cudaError_t lbm_tma_build(const float *g0, const float *g1, const float2 *force, int nx, int ny,
-                          int nmem, LbmTma *out) {
-    out->ok = 0;
-    constexpr int AX = kTX + 8, AY = kTY + 4;
-    static_assert(2 * AX <= 256 && AY <= 256 && NV <= 256, "a TMA box has at most 256 per side");
-    if ((nx & 3) != 0 || nx < AX || ny < AY || nmem <= 0) return cudaSuccess;   // cp.async only
-    // without the driver's encoder the staging stays on cp.async (the same values); a map the
-    // encoder rejects is an error
-    const EncodeTiled enc = encode_tiled();
-    if (!enc) return cudaSuccess;
-    const cuuint32_t es[3] = {1, 1, 1};
-    // state [nmem * 9 planes][ny][nx] floats; box: one member's nine planes of the window
-    const cuuint64_t gdim[3] = {(cuuint64_t)nx, (cuuint64_t)ny, (cuuint64_t)nmem * NV};
-    const cuuint64_t gstr[2] = {(cuuint64_t)nx * 4, (cuuint64_t)nx * ny * 4};
-    const cuuint32_t gbox[3] = {AX, AY, NV};
-    for (int b = 0; b < 2; ++b)
-        if (enc(reinterpret_cast<CUtensorMap *>(&out->g[b]), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
-                const_cast<float *>(b ? g1 : g0), gdim, gstr, gbox, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
-    out->gptr[0] = g0;
-    out->gptr[1] = g1;
-    out->ok = 1;
-    if (force) {   // [ny][2 nx] floats (the components interleaved); box: the window's rows
-        const cuuint64_t fdim[2] = {(cuuint64_t)2 * nx, (cuuint64_t)ny};
-        const cuuint64_t fstr[1] = {(cuuint64_t)2 * nx * 4};
-        const cuuint32_t fbox[2] = {2 * AX, AY};
-        if (enc(reinterpret_cast<CUtensorMap *>(&out->f), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
-                const_cast<float2 *>(force), fdim, fstr, fbox, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
-        out->ok |= 2;
+#define LK_STEPS(T)                                                                             \
+    case T:                                                                                     \
+        return force ? launch_steps<T, true>(gin, gout, force, nx, ny, nmem, tau, s, rows[T - 1]) \
+                     : launch_steps<T, false>(gin, gout, force, nx, ny, nmem, tau, s, rows[T - 1]);
+    switch (steps) {
+        LK_STEPS(1)
+        LK_STEPS(2)
+        LK_STEPS(3)
+        LK_STEPS(4)
+        default: return cudaErrorInvalidValue;
     }
-    return cudaSuccess;
+#undef LK_STEPS
 }
 
 cudaError_t launch_f_to_g(const float *f, float *g, int nmem, size_t npts, cudaStream_t s) {
