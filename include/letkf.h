@@ -67,7 +67,10 @@ extern "C" {
 /* Eigensolve schedules (same results up to rounding; see letkf_config.eig_schedule). */
 #define LETKF_EIG_AUTO        0  /* the handle picks one: at its first analysis the schedules
                                     (FUSED, SPLIT and, for k <= 64, CHEBYSHEV, which passes its
-                                    ill-conditioned points to RATIONAL) are timed on
+                                    ill-conditioned points to RATIONAL; for k > 64, on chunks of
+                                    4,096 points and more, SPLIT with CHEBYSHEV's transform
+                                    before it for the points with kappa up to 400, named SPLIT in
+                                    letkf_stats) are timed on
                                     that analysis' first chunk of Gram matrices
                                     (applied to a scratch copy of the forecast, so the analysis
                                     itself is unaffected; one host synchronisation), and the
@@ -421,7 +424,7 @@ double letkf_chebyshev_coefficients(double kappa_max, int32_t n, double *c_rsqrt
 /* Cumulative counts of the LETKF_EIG_CHEBYSHEV transform on this handle since letkf_init
  * (device counters, also advanced by the AUTO tuner's trial runs): counts[0] grid points
  * transformed, counts[1] products with A formed (the sum of the degrees used), counts[2]
- * points passed on to the RATIONAL schedule.  Waits for the handle's stream; LETKF_EINVAL for
+ * points passed on to the RATIONAL (for k > 64 the SPLIT) schedule.  Waits for the handle's stream; LETKF_EINVAL for
  * NULL arguments. */
 int letkf_get_work_counts(letkf_handle *h, int64_t *counts);
 

@@ -37,6 +37,13 @@ constexpr int64_t kDefaultChunkBytes = 1ll << 30;  // 1 GiB: 65,536 points at k 
 constexpr int64_t kGemmMaxBytes = 2ll << 30;
 constexpr int kGemmMinPoints = 1024;
 
+// AUTO at k > 64 puts the polynomial transform before the split schedule on chunks of this many
+// points.  It is the faster at every size (k = 80 / 128, kappa some tens: 32 x 32 points 0.16 /
+// 0.20 ms against 0.68 / 4.2 of the better other one, 64 x 64 0.60 / 0.72 against 3.3 / 13.6,
+// 96 x 96 1.2 / 1.5 against 6.6 / 30.9); smaller chunks keep to the schedules that a
+// configuration can name at these k, so that naming AUTO's pick repeats its run bit for bit there.
+constexpr int kChebAutoMinPoints = 4096;
+
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 int kp_of(int k) { return k <= 8 ? 8 : k <= 16 ? 16 : k <= 32 ? 32 : k <= 64 ? 64 : 128; }
@@ -213,9 +220,8 @@ int make_plan(const letkf_config *c, Plan *p) {
     p->off_rot = take(record ? p->chunk_pts * (size_t)p->rcap * sizeof(float2) : 0);
     p->off_nrot = take(record ? p->chunk_pts * sizeof(int) : 0);
     p->off_list = take(split ? (p->chunk_pts + 4) * sizeof(int) : 0);
-    // the Chebyshev transform's hand-off list (CHEBYSHEV, and AUTO where it is a candidate)
-    const bool cheb = (p->eig_schedule == LETKF_EIG_CHEBYSHEV ||
-                       p->eig_schedule == LETKF_EIG_AUTO) && c->k <= lk::kChebMaxK;
+    // the Chebyshev transform's hand-off list (CHEBYSHEV, and AUTO, which may pick it)
+    const bool cheb = p->eig_schedule == LETKF_EIG_CHEBYSHEV || p->eig_schedule == LETKF_EIG_AUTO;
     p->off_pre_list = take(cheb ? (p->chunk_pts + 4) * sizeof(int) : 0);
     p->off_status = take(kAlign);
     p->total = align_up(off, kAlign);
@@ -482,16 +488,17 @@ lk::EigArgs eig_args(letkf_handle *h, int y0, int y1) {
     return e;
 }
 
-// The EVD-free schedules serve k <= 64; AUTO considers them there.  The Chebyshev schedule
-// hands the points beyond its approximations to the rational one, which it therefore needs.
+// The EVD-free schedules serve k <= 64; AUTO considers them there.  The Chebyshev schedule hands
+// the points beyond its approximations to the rational one, which it therefore needs.  For
+// k > 64, where a configuration cannot name it, AUTO considers it on chunks of kChebAutoMinPoints
+// and more; there it hands the points beyond to the split schedule (whose scratch AUTO has).
 bool rational_candidate(int schedule, int k) {
     return (schedule == LETKF_EIG_RATIONAL || schedule == LETKF_EIG_CHEBYSHEV ||
             schedule == LETKF_EIG_AUTO) &&
            k <= lk::kRationalMaxK;
 }
-bool cheb_candidate(int schedule, int k) {
-    return (schedule == LETKF_EIG_CHEBYSHEV || schedule == LETKF_EIG_AUTO) &&
-           k <= lk::kChebMaxK;
+bool cheb_candidate(int schedule) {
+    return schedule == LETKF_EIG_CHEBYSHEV || schedule == LETKF_EIG_AUTO;
 }
 
 // The chunk's eigensolve, transform and update on the handle's resolved schedule.
@@ -504,6 +511,10 @@ cudaError_t launch_eig_schedule(letkf_handle *h, int schedule, lk::EigArgs e, cu
     if (schedule == LETKF_EIG_RATIONAL) {
         e.eigval = want_eigval ? h->eigval : nullptr;
         return lk::launch_eigen_rational(e, h->eig_split, h->rat_grid, s);
+    }
+    if (schedule == LETKF_EIG_CHEBYSHEV && h->cfg.k > lk::kChebMaxK) {
+        e.eigval = h->eigval;
+        return lk::launch_eigen_cheb_split(e, h->eig_split, h->cheb_grid, want_eigval, s);
     }
     if (schedule == LETKF_EIG_CHEBYSHEV) {
         e.eigval = want_eigval ? h->eigval : nullptr;
@@ -545,10 +556,17 @@ int cached_eig_schedule(const letkf_handle *h) {
     return it == c.pick.end() ? LETKF_EIG_AUTO : it->second;
 }
 
+// What letkf_stats names: a schedule that a configuration of this k may name too.
+int reported_schedule(const letkf_handle *h) {
+    return h->eig_schedule == LETKF_EIG_CHEBYSHEV && h->cfg.k > lk::kChebMaxK ? LETKF_EIG_SPLIT
+                                                                             : h->eig_schedule;
+}
+
 int tune_eig_schedule(letkf_handle *h, int y0, int y1) {
     const int cached = cached_eig_schedule(h);
     if (cached != LETKF_EIG_AUTO) {
-        h->eig_schedule = h->stats.eig_schedule = cached;
+        h->eig_schedule = cached;
+        h->stats.eig_schedule = reported_schedule(h);
         return LETKF_OK;
     }
     const int k = h->cfg.k;
@@ -568,9 +586,10 @@ int tune_eig_schedule(letkf_handle *h, int y0, int y1) {
     // point beyond its break-even degree to the rational one, so it is never much slower than
     // that, and timing the two on the first analysis (whose spread may be far from the later
     // ones') would tie the process to a transient
-    int cand[3] = {LETKF_EIG_FUSED, LETKF_EIG_SPLIT, 0};
-    int ncand = 2;
-    if (cheb_candidate(LETKF_EIG_AUTO, k)) cand[ncand++] = LETKF_EIG_CHEBYSHEV;
+    // (and for k > 64 it stands for the split schedule, which gets the points beyond)
+    int cand[3] = {LETKF_EIG_FUSED, LETKF_EIG_SPLIT, LETKF_EIG_CHEBYSHEV};
+    int ncand = k <= lk::kChebMaxK ? 3 : 2;
+    if (k > lk::kChebMaxK && e.npts >= kChebAutoMinPoints) cand[1] = LETKF_EIG_CHEBYSHEV;
     float best[3] = {0.0f, 0.0f, 0.0f};
     cudaError_t err = cudaEventCreate(&t0);
     if (err == cudaSuccess) err = cudaEventCreate(&t1);
@@ -600,7 +619,7 @@ int tune_eig_schedule(letkf_handle *h, int y0, int y1) {
         std::lock_guard<std::mutex> lock(c.mu);
         h->eig_schedule = c.pick.emplace(eig_tune_key(h), pick).first->second;  // first wins
     }
-    h->stats.eig_schedule = h->eig_schedule;
+    h->stats.eig_schedule = reported_schedule(h);
     return LETKF_OK;
 }
 
@@ -1067,7 +1086,7 @@ int letkf_init(const letkf_config *cfg, void *workspace, size_t workspace_bytes,
         h->eig_split.nrot = plan.rcap > 0 ? (int *)(w + plan.off_nrot) : nullptr;
         h->eig_split.list = (int *)(w + plan.off_list);
         h->eig_split.list_count = h->eig_split.list + plan.chunk_pts;
-        if (cheb_candidate(plan.eig_schedule, cfg->k)) {
+        if (cheb_candidate(plan.eig_schedule)) {
             h->eig_split.pre_list = (int *)(w + plan.off_pre_list);
             h->eig_split.pre_count = h->eig_split.pre_list + plan.chunk_pts;
         }
@@ -1137,7 +1156,7 @@ int letkf_init(const letkf_config *cfg, void *workspace, size_t workspace_bytes,
          lk::eigen_split_prepare(cfg->k, &h->eig_split) != cudaSuccess) ||
         (rational_candidate(plan.eig_schedule, cfg->k) &&
          lk::eigen_rational_prepare(cfg->k, &h->rat_grid) != cudaSuccess) ||
-        (cheb_candidate(plan.eig_schedule, cfg->k) &&
+        (cheb_candidate(plan.eig_schedule) &&
          lk::eigen_cheb_prepare(cfg->k, &h->cheb_grid) != cudaSuccess))
         return fail(LETKF_ECUDA);
     if (plan.gemm) {
@@ -1190,7 +1209,7 @@ int letkf_init(const letkf_config *cfg, void *workspace, size_t workspace_bytes,
     // AUTO: the process' earlier pick for this shape, else timed at the first analysis
     h->eig_schedule =
         plan.eig_schedule == LETKF_EIG_AUTO ? cached_eig_schedule(h) : plan.eig_schedule;
-    h->stats.eig_schedule = h->eig_schedule;
+    h->stats.eig_schedule = reported_schedule(h);
     // the Gram: tensor cores (mixed), the one team schedule (k <= 16), else as configured
     if (plan.tensor_gram || h->gemm)
         h->gram_tile = LETKF_GRAM_TENSOR;

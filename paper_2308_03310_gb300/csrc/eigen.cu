@@ -1346,19 +1346,24 @@ __global__ void __launch_bounds__(32 * kPairWarps, 5) eig_tridiag_pair_kernel(Ei
 // kept in shared memory as [index][thread] (the threads of a warp touch consecutive words),
 // every rotation recorded.  Record of a point: per sweep a header (m, count) -- bit patterns
 // of two ints -- then the sweep's (c, s) for i = m-1 down to m-count.
+// kList: only the listed points.
+template <bool kList>
 __global__ void __launch_bounds__(kQlThreads) eig_ql_kernel(EigArgs a, EigSplit sp) {
     extern __shared__ float2 des[];  // [k][kQlThreads]
     const int k = a.k, tid = threadIdx.x;
     const int lp0 = blockIdx.x * kQlThreads;
-    const int lp = lp0 + tid;
-    // the block's (d, e) arrays are contiguous in global memory: coalesced load
-    const int nb = min(kQlThreads, a.npts - lp0);
+    const int npts = kList ? *a.list_count : a.npts;
+    // the block's (d, e) arrays are contiguous in global memory (a listed point's is): coalesced
+    // load
+    const int nb = min(kQlThreads, npts - lp0);
     for (int e = tid; e < nb * k; e += kQlThreads) {
         const int p = e / k, i = e - p * k;
-        des[i * kQlThreads + p] = sp.de[(size_t)lp0 * k + e];
+        des[i * kQlThreads + p] =
+            kList ? sp.de[(size_t)a.list[lp0 + p] * k + i] : sp.de[(size_t)lp0 * k + e];
     }
     __syncthreads();
-    if (lp >= a.npts) return;
+    if (tid >= nb) return;
+    const int lp = kList ? a.list[lp0 + tid] : lp0 + tid;
     if (a.nloc && a.nloc[lp] == 0) {
         for (int t = 0; t < k; ++t) a.eigval[(size_t)lp * k + t] = a.diag;
         if (sp.nrot) sp.nrot[lp] = 0;
@@ -1612,7 +1617,7 @@ __device__ __forceinline__ void replay_in_registers(const float2 *__restrict__ r
 // onto Z, V = H Z, then the fused schedule's transform and update (kUpdate; without it, the
 // eigenpairs only, for letkf_eigh_batch_ws: a separate instantiation, so that the analysis
 // path carries no extra registers).
-template <int NC, bool kUpdate>
+template <int NC, bool kUpdate, bool kList = false>
 __global__ void __launch_bounds__(32 * EigCfg<NC>::WARPS, EigCfg<NC>::MINB_VEC)
     eig_vec_kernel(EigArgs a, EigSplit sp) {
     extern __shared__ float smem[];
@@ -1624,7 +1629,9 @@ __global__ void __launch_bounds__(32 * EigCfg<NC>::WARPS, EigCfg<NC>::MINB_VEC)
     float *taus = B + kRows * ld;
     const int warps_per_block = blockDim.x >> 5;
     const int nw = gridDim.x * warps_per_block;
-    for (int lp = blockIdx.x * warps_per_block + wib; lp < a.npts; lp += nw) {
+    const int npts = kList ? *a.list_count : a.npts;   // the listed points, or the chunk
+    for (int it = blockIdx.x * warps_per_block + wib; it < npts; it += nw) {
+        const int lp = kList ? a.list[it] : it;
         const int nrec = sp.nrot[lp];
         if (a.nloc && a.nloc[lp] == 0) {  // no local observation: Q = (k-1)/rho I
             if constexpr (kUpdate) inflate_point(a, lp, lane);
@@ -1766,7 +1773,16 @@ cudaError_t prepare_split_nc(int k, EigSplit *sp) {
                       (size_t)vec_smem_floats(k) * sizeof(float) * warps,
                       (size_t)vec_smem_floats(kmax_of(NC)) * sizeof(float) * warps, &unused);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(eig_ql_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if constexpr (NC == 4) {
+        e = occupancy<NC>((const void *)eig_vec_kernel<NC, true, true>, warps,
+                          (size_t)vec_smem_floats(k) * sizeof(float) * warps,
+                          (size_t)vec_smem_floats(kmax_of(NC)) * sizeof(float) * warps, &unused);
+        if (e != cudaSuccess) return e;
+    }
+    e = cudaFuncSetAttribute(eig_ql_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(128 * kQlThreads * sizeof(float2)));
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(eig_ql_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)(128 * kQlThreads * sizeof(float2)));
 }
 
@@ -1818,13 +1834,23 @@ void launch_tri(const EigArgs &a, const EigSplit &sp, cudaStream_t s) {
 }
 
 void launch_ql(const EigArgs &a, const EigSplit &sp, cudaStream_t s) {
-    eig_ql_kernel<<<(unsigned)((a.npts + kQlThreads - 1) / kQlThreads), kQlThreads,
-                    (size_t)a.k * kQlThreads * sizeof(float2), s>>>(a, sp);
+    const unsigned blocks = (unsigned)((a.npts + kQlThreads - 1) / kQlThreads);
+    const size_t smem = (size_t)a.k * kQlThreads * sizeof(float2);
+    if (a.list) eig_ql_kernel<true><<<blocks, kQlThreads, smem, s>>>(a, sp);
+    else eig_ql_kernel<false><<<blocks, kQlThreads, smem, s>>>(a, sp);
 }
 
 template <int NC>
 void launch_vec(const EigArgs &a, const EigSplit &sp, cudaStream_t s) {
     const int warps = EigCfg<NC>::WARPS;
+    if constexpr (NC == 4) {   // k > 64: the points that the Chebyshev transform handed on
+        if (a.list) {
+            eig_vec_kernel<NC, true, true><<<grid_for(sp.grid_vec, a.npts, warps), 32 * warps,
+                                             (size_t)vec_smem_floats(a.k) * sizeof(float) * warps,
+                                             s>>>(a, sp);
+            return;
+        }
+    }
     if (a.x)
         eig_vec_kernel<NC, true><<<grid_for(sp.grid_vec, a.npts, warps), 32 * warps,
                                    (size_t)vec_smem_floats(a.k) * sizeof(float) * warps, s>>>(a,
@@ -1870,7 +1896,7 @@ cudaError_t launch_split_nc(const EigArgs &a, const EigSplit &sp, cudaStream_t s
         launch_ql(a, sp, s);
         launch_vec<NC>(a, sp, s);
     }
-    // matrices whose rotation record overflowed: the fused kernel over the list
+    // matrices whose rotation record overflowed: the fused kernel over its list
     EigArgs f = a;
     f.list = sp.list;
     f.list_count = sp.list_count;
@@ -2016,6 +2042,29 @@ cudaError_t launch_eigen_chebyshev(const EigArgs &a, const EigSplit &sp, int che
     if (a.k <= 32) return launch_rational_nc<1>(r, sp, rat_grid, s);
     if (a.k <= kChebMaxK) return launch_rational_nc<2>(r, sp, rat_grid, s);
     return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_eigen_cheb_split(const EigArgs &a, const EigSplit &sp, int cheb_grid,
+                                    bool want_eigval, cudaStream_t s) {
+    if (a.npts <= 0) return cudaSuccess;
+    if (a.k <= kChebMaxK || a.k > kChebSplitMaxK || !a.eigval || !sp.de || !sp.taus || !sp.rot ||
+        !sp.nrot || !sp.list || !sp.list_count || !sp.pre_list || !sp.pre_count || !a.x ||
+        !a.cvec || a.list)
+        return cudaErrorInvalidValue;
+    cudaError_t e = cudaMemsetAsync(sp.pre_count, 0, sizeof(int), s);
+    if (e != cudaSuccess) return e;
+    if (want_eigval) {   // the QL without a record; the upper triangles stay as they are
+        EigSplit v = sp;
+        v.rot = nullptr;
+        v.nrot = nullptr;
+        launch_tri<4>(a, v, s);
+        launch_ql(a, v, s);
+    }
+    if ((e = launch_eigen_cheb_transform(a, sp, cheb_grid, s)) != cudaSuccess) return e;
+    EigArgs r = a;
+    r.list = sp.pre_list;
+    r.list_count = sp.pre_count;
+    return launch_split_nc<4>(r, sp, s, nullptr, nullptr, nullptr);
 }
 
 cudaError_t launch_eigen_split(const EigArgs &a, const EigSplit &sp, cudaStream_t s,

@@ -136,8 +136,8 @@ struct EigArgs {
     float *eigval = nullptr;        // [npts][k] eigenvalues; optional for the fused schedule
     int *status = nullptr;          // device status word
     int max_blocks = 0;             // resident grid of the fused kernel (eigen_prepare)
-    const int *list = nullptr;      // only these points (count in *list_count): the fused
-    const int *list_count = nullptr;  // kernel, the tridiagonalizations, the rational transform
+    const int *list = nullptr;      // only these points (count in *list_count): the fused and
+    const int *list_count = nullptr;  // split kernels, the rational transform
     float *evec = nullptr;          // optional [npts][k][k]: row i = eigenvector of eigval[i]
     int refine = 0;                 // FP64 refinement sweep of clustered eigenpairs
     float refine_tau = 0.0f;        // relative eigenvalue distance that makes a cluster
@@ -202,13 +202,17 @@ cudaError_t launch_eigen_rational(const EigArgs &a, const EigSplit &sp, int grid
 // condition bound is used.
 constexpr int kChebSets = 15;
 constexpr int kChebMaxDeg = 36;
-constexpr int kChebMaxK = 64;
+constexpr int kChebMaxK = 64;       // LETKF_EIG_CHEBYSHEV; beyond, up to kChebSplitMaxK, AUTO may
+constexpr int kChebSplitMaxK = 128;  // choose it, with the sets up to kappa 400
+constexpr int kChebBigSets = 23;
+constexpr int kChebCoefs = 1100;
 struct ChebTable {
-    float kappa_max[kChebSets];
-    int n[kChebSets];                        // degree
-    float2 c[kChebSets][kChebMaxDeg + 1];    // (t^-1/2, t^-1) coefficients of T_0 .. T_n
+    float kappa_max[kChebBigSets];
+    int n[kChebBigSets];            // degree
+    int off[kChebBigSets];          // the set's first coefficient
+    float2 c[kChebCoefs];           // (t^-1/2, t^-1) coefficients of T_0 .. T_n per set
 };
-const ChebTable &cheb_table();              // computed once per process (chebyshev.cu)
+const ChebTable &cheb_table(int k);         // computed once per process (chebyshev.cu)
 int cheb_max_set(int k);                    // the largest set used at ensemble size k
 double chebyshev_coefficients(double kappa, int n, double *ca, double *cb);
 cudaError_t eigen_cheb_prepare(int k, int *grid);
@@ -219,6 +223,11 @@ cudaError_t launch_eigen_cheb_transform(const EigArgs &a, const EigSplit &sp, in
 // handed on (sp needs de, taus, list, list_count, pre_list and pre_count)
 cudaError_t launch_eigen_chebyshev(const EigArgs &a, const EigSplit &sp, int cheb_grid,
                                    int rat_grid, cudaStream_t s);
+
+// k > kChebMaxK: the Chebyshev transform, then the split schedule over the points it handed on
+// (needs a.eigval and the rotation record too); with want_eigval every point's eigenvalues
+cudaError_t launch_eigen_cheb_split(const EigArgs &a, const EigSplit &sp, int cheb_grid,
+                                    bool want_eigval, cudaStream_t s);
 
 cudaError_t eigen_prepare(int k, int *max_blocks);  // once per process and k
 cudaError_t eigen_split_prepare(int k, EigSplit *sp);
