@@ -33,10 +33,10 @@
 //   warps 8..15  sums: tensor memory added into registers per step, then stored to the Gram
 //                slots and c in global memory
 // Measured (Gram phase, z included): 1024^2, k = 64, r = 12, every fourth point observed 93.7 ms ->
-// 15.5 ms (CUDA cores in FP32; the split-FP16 tensor form 48.4 ms); 256^2, k = 32, r = 8, every
-// eighth point 0.393 -> 0.117 ms; 250 x 187, k = 40, three variables, Gaspari-Cohn 2.16 -> 0.33 ms.
+// 15.05 ms (CUDA cores in FP32; the split-FP16 tensor form 48.4 ms); 256^2, k = 32, r = 8, every
+// eighth point 0.393 -> 0.110 ms; 250 x 187, k = 40, three variables, Gaspari-Cohn 2.16 -> 0.33 ms.
 // Relative error of A against 64 bits (256^2, k = 64, spread 5e-3): 4.2e-7 -> 1.8e-7.  The tensor
-// pipe needs about 8 ms of the 15.5 (18 pair tiles x 20 steps x 12 MMAs of 128 cycles per tile);
+// pipe needs about 8 ms of the 15.05 (18 pair tiles x 20 steps x 12 MMAs of 128 cycles per tile);
 // the weights' FP32 work (about 1,000 issue slots per scheduler and step) bounds it next.
 // Every wait is bounded in time: on expiry the status word gets ST_TIMEOUT, all roles leave, the
 // copies and MMAs in flight are awaited (bounded) and the tensor memory is freed.
@@ -70,9 +70,10 @@ constexpr int kWSbo = (kKC / 8) * 128;         // bytes between 8-point core blo
 constexpr int kThreads = 512;
 constexpr int kWarpMeta = 0, kWarpTma = 1, kWarpMma = 2, kWarpProd = 4, kWarpSum = 8;
 constexpr int kProdWarps = 4, kSumWarps = 8;
-// registers per thread of the three roles (setmaxnreg): the sums hold 128 accumulators; the
-// block is launched with 512 x 128
-constexpr int kRegMisc = 56, kRegProd = 88, kRegSum = 184;
+// registers per thread of the three roles (setmaxnreg): the sums hold 128 accumulators and read
+// 16 columns at a time (32 would take 184 and leave the weights' warps 88: 15.5 ms against 15.05);
+// the block is launched with 512 x 128
+constexpr int kRegMisc = 56, kRegProd = 120, kRegSum = 168;
 static_assert(kRegMisc + kRegProd + 2 * kRegSum <= 4 * 128, "the launch's registers");
 constexpr uint32_t kCols = 512;
 
@@ -571,11 +572,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!(ok = wait_bar(&tm_full[tb], (g >> 1) & 1, &abort_flag))) break;
                 asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
-                for (int c = 0; c < kPts / 2; c += 32) {
-                    float v[32];
-                    tmem_ld32(src + tb * kPts + c, v);
+                for (int c = 0; c < kPts / 2; c += 16) {
+                    float v[16];
+                    tmem_ld16(src + tb * kPts + c, v);
 #pragma unroll
-                    for (int i = 0; i < 32; i += 2) {
+                    for (int i = 0; i < 16; i += 2) {
                         const float2 t = __fadd2_rn(make_float2(acc[c + i], acc[c + i + 1]),
                                                     make_float2(v[i], v[i + 1]));
                         acc[c + i] = t.x;
