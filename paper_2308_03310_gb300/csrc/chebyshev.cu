@@ -23,12 +23,15 @@
 // approximation goes to the rational schedule (tridiagonalization and Zolotarev's
 // approximation) through a list.
 //
-// Layout: A in registers, 32 rows of two columns per lane (one column for k <= 32), loaded from
-// the upper triangle of the Gram slot staged in shared memory; one warp per grid point for
-// k <= 32, two (halves of the rows) for k <= 64, eight (quarters of the rows x halves of the
-// columns) for k <= 128, so that 16 warps or more share an SM.  A product R A reads the rows of R
-// as 16-byte broadcasts (five loads for 20 packed multiply-adds) and the warps' partial sums
-// meet in shared memory; the recurrence's own values stay in registers.
+// Layout, k <= 64 (eig_cheb_kernel): one warp per grid point.  A half warp holds half of the rows of
+// A in registers, a lane four columns (two for k <= 32), loaded from the upper triangle of the Gram
+// slot staged in shared memory.  A product R A reads the rows of R as 16-byte broadcasts to a half
+// warp (five loads for 40 packed multiply-adds) and ends with a shuffle between the half warps.
+// The rows of R are independent: five run through the whole recurrence, its values in
+// registers, then the other five.  (Broadcasts to a whole warp took twice the shared-memory
+// wavefronts, and two warps per point, halves of the rows, 1.5 times the instructions.)
+// k <= 128 (eig_cheb_block_kernel): eight warps per point, quarters of the rows x halves of the
+// columns, 32 rows of two columns per lane; the partial sums meet in shared memory.
 #include <math.h>
 
 #include <algorithm>
@@ -158,27 +161,37 @@ namespace {
 constexpr unsigned kAllC = 0xffffffffu;
 constexpr int kRowsC = 10;   // rows of R: the nine populations' perturbations, then c
 
-template <int KM>
-struct ChebShape {
-    static constexpr int NW = KM == 32 ? 1 : KM == 64 ? 2 : 8;   // warps per point
-    static constexpr int PPB = NW == 1 ? 4 : 1;                  // points per block
+// Eight warps per point (k <= 128).
+struct ChebBlock {
+    static constexpr int KM = 128, NW = 8;                       // warps per point
     static constexpr int CS = KM / 32;                           // 32-column slots of a row
-    static constexpr int NC = KM == 32 ? 1 : 2;                  // columns of a lane
+    static constexpr int NC = 2;                                 // columns of a lane
     static constexpr int CG = CS / NC, RB = NW / CG;             // column groups, row blocks
-    static constexpr int RR = KM / RB;                           // rows of a block
     static constexpr int NE = kRowsC * CS / NW;                  // (row, slot) entries of a warp
     static constexpr int SP = KM + 4;                            // stride of the staged slot
     static constexpr int off_x = KM * SP;                        // [9][k] and c[k]
     static constexpr int off_b = off_x + kRowsC * KM;            // b_{j+1}, [10][KM]
     static constexpr int off_p = off_b + kRowsC * KM;            // partial sums
-    static constexpr int psize = RB == 1 ? KM : RB == 2 ? kRowsC * KM : RB * kRowsC * KM;
-    static constexpr int off_r = off_p + psize;                  // reductions over the warps
-    static constexpr int floats = off_r + 2 * NW + 2 * kRowsC * CS + (KM == 32 ? 6 : 0);
-    static_assert(RR == 32 && psize >= RB * KM, "32 rows per block; the columns' sums fit");
-    static_assert(floats % 4 == 0, "16-byte aligned point buffers");
-    // blocks per SM: 12 warps with 168 registers (k <= 64; 16 warps of 128 spill and measured 8 %
-    // slower at k = 64, 6 % at k = 32), 16 with 128 (k <= 128, by shared memory)
-    static constexpr int MINB = KM == 32 ? 3 : KM == 64 ? 6 : 2;
+    static constexpr int off_r = off_p + RB * kRowsC * KM;       // reductions over the warps
+    static constexpr int floats = off_r + 2 * NW + 2 * kRowsC * CS;
+    static_assert(KM == 32 * RB && floats % 4 == 0, "32 rows per block, 16-byte aligned buffers");
+};
+
+// One warp per point, kWarpsC points per block.
+constexpr int kWarpsC = 4;
+template <int KM>
+struct ChebShape {
+    static constexpr int NC = KM / 16, HC = NC / 2;   // columns of a lane; kept after a product
+    static constexpr int RH = KM / 2;                 // rows of a half warp
+    static constexpr int SP = KM + 4;                 // stride of the staged slot
+    static constexpr int off_x = KM * SP;             // [9][k] and c[k]
+    static constexpr int off_r = off_x + kRowsC * KM; // rows 0..4, kept for the second pass
+    static constexpr int off_b = off_r + 5 * KM;      // b_{j+1}, [5][KM]
+    static constexpr int off_u = off_b + 5 * KM;      // Q^-1 c
+    static constexpr int floats = off_u + KM;
+    static_assert(floats % 4 == 0 && off_b % 4 == 0, "16-byte aligned buffers");
+    // blocks per SM: 8 warps with 255 registers (128 of them A), 16 with 128
+    static constexpr int MINB = KM == 32 ? 4 : 2;
 };
 
 constexpr unsigned long long kChebWaitNs = 2000000000ull;   // bound of a prefetch wait (2 s)
@@ -207,19 +220,338 @@ __device__ __forceinline__ float warp_max_c(float v) {
     return v;
 }
 
-template <int NW>
-__device__ __forceinline__ void point_sync() {   // the warps of one point
-    if constexpr (NW == 1) __syncwarp();
-    else __syncthreads();
+// Five rows of R (b, row stride KM, this half warp's first row of A) times NG groups of four rows of
+// A per half warp; sums over both half warps, each lane keeping half of its columns.  (With a
+// run-time bound on the groups every group waited for its own loads.)
+template <int KM, int NG>
+__device__ __forceinline__ void cheb_product_ng(
+    const float *b, const float2 (&A)[ChebShape<KM>::NC][ChebShape<KM>::RH / 2], int half,
+    float (&out)[5][ChebShape<KM>::HC]) {
+    constexpr int NC = ChebShape<KM>::NC, HC = NC / 2;
+    const float4 *B4 = reinterpret_cast<const float4 *>(b);
+    float2 acc[5][NC];
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+#pragma unroll
+        for (int rr = 0; rr < 5; ++rr) {
+            const float4 v = B4[rr * (KM / 4) + g];
+#pragma unroll
+            for (int q = 0; q < NC; ++q)
+                acc[rr][q] = g ? __ffma2_rn(make_float2(v.x, v.y), A[q][2 * g], acc[rr][q])
+                               : __fmul2_rn(make_float2(v.x, v.y), A[q][0]);
+#pragma unroll
+            for (int q = 0; q < NC; ++q)
+                acc[rr][q] = __ffma2_rn(make_float2(v.z, v.w), A[q][2 * g + 1], acc[rr][q]);
+        }
+#pragma unroll
+    for (int rr = 0; rr < 5; ++rr)
+#pragma unroll
+        for (int q = 0; q < HC; ++q) {
+            const float lo = acc[rr][q].x + acc[rr][q].y;
+            const float hi = acc[rr][HC + q].x + acc[rr][HC + q].y;
+            out[rr][q] = (half ? hi : lo) + __shfl_xor_sync(kAllC, half ? lo : hi, 16);
+        }
+}
+
+template <int KM>
+__device__ __forceinline__ void cheb_product(
+    const float *b, const float2 (&A)[ChebShape<KM>::NC][ChebShape<KM>::RH / 2], int ng, int half,
+    float (&out)[5][ChebShape<KM>::HC]) {
+    if constexpr (KM == 64) {   // k > 32: 5 to 8 groups
+        if (ng > 7) cheb_product_ng<KM, 8>(b, A, half, out);
+        else if (ng > 6) cheb_product_ng<KM, 7>(b, A, half, out);
+        else if (ng > 5) cheb_product_ng<KM, 6>(b, A, half, out);
+        else cheb_product_ng<KM, 5>(b, A, half, out);
+    } else {
+        if (ng > 3) cheb_product_ng<KM, 4>(b, A, half, out);
+        else if (ng > 2) cheb_product_ng<KM, 3>(b, A, half, out);
+        else cheb_product_ng<KM, 2>(b, A, half, out);
+    }
+}
+
+// k <= 64.  What bounds it: 10 k^2 multiply-adds per product and point on the FP32 pipe, at two warps
+// per scheduler (k <= 32: four), and before the products the assembly of A from the staged
+// triangle (about two products' time at k = 64).  Eigensolve phase, two warps per point -> this form:
+// 256 x 256, k = 64, 28.4 products a point 4.23 -> 3.83 ms; 1024 x 1024, k = 64, three products
+// 13.7 -> 11.9 ms; 250 x 187, k = 40, 20.7 products 2.01 -> 1.67 ms; one warp per point with
+// broadcasts to the whole warp -> this form: 256 x 256, k = 32, 5.8 products 0.378 -> 0.358 ms;
+// 301 x 215, k = 24, 9.7 products 0.436 -> 0.414 ms.
+template <int KM>
+__global__ void __launch_bounds__(32 * kWarpsC, ChebShape<KM>::MINB)
+    eig_cheb_kernel(EigArgs a, EigSplit sp, const __grid_constant__ ChebTable ct, int max_set) {
+    using S = ChebShape<KM>;
+    constexpr int NC = S::NC, HC = S::HC, SP = S::SP;
+    extern __shared__ float4 smem_c4[];
+    __shared__ __align__(8) uint64_t pbar[kWarpsC];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    float *G = reinterpret_cast<float *>(smem_c4) + (size_t)wib * S::floats;
+    float *XS = G + S::off_x, *RS = G + S::off_r, *B = G + S::off_b, *U = G + S::off_u;
+    const int k = a.k;
+    const float d = a.diag, inv_d = 1.0f / a.diag;
+    const float sc = sqrtf((float)(k - 1)) / sqrtf(a.diag);   // sqrt(k-1) d^-1/2
+    const int half = lane >> 4, cj = 2 * (lane & 15);         // columns cj, cj + 1 (+ 32, + 33)
+    const int col = KM == 64 ? 32 * half + cj : cj + half;    // of them this lane's own: col (, + 1)
+    const int ng = (k + 7) / 8, row0 = 4 * ng * half;         // groups of four rows per half warp
+    unsigned long long n_pts = 0, n_prod = 0, n_hand = 0;
+    const long long nw = (long long)gridDim.x * kWarpsC;
+    // Where the Gram slot's rows are 16-byte multiples (k a multiple of 4) the next point's upper
+    // triangle (bulk copies of every row from its first multiple of 4), forecast block and c are
+    // fetched into the stage while this point is worked on, counted in bytes on the warp's
+    // mbarrier; otherwise the warp loads them when the point begins.
+    const bool pf = (k & 3) == 0;
+    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&pbar[wib]);
+    uint32_t phase = 0;
+    auto bulk = [&](float *dst, const float *src, int n) {
+        asm volatile(
+            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, "
+            "[%3];" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+            "l"(src), "r"((uint32_t)(n * 4)), "r"(bar)
+            : "memory");
+    };
+    auto prefetch = [&](long long q) {
+        const int g = k / 4;
+        if (lane == 0)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                         "r"((uint32_t)((8 * g * (g + 1) + kRowsC * k) * 4))
+                         : "memory");
+        __syncwarp();
+        const float *src = a.gram + (size_t)q * k * k;
+        for (int i = lane; i < k; i += 32)
+            bulk(G + i * SP + (i & ~3), src + (size_t)i * k + (i & ~3), k - (i & ~3));
+        if (lane == 0) bulk(XS, a.x + (size_t)(a.pt0 + q) * NV * k, NV * k);
+        if (lane == 1) bulk(XS + NV * k, a.cvec + (size_t)q * k, k);
+    };
+    // the stage is zero beyond k rows and columns throughout
+    for (int e = lane; e < S::floats; e += 32) G[e] = 0.0f;
+    if (lane == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    long long lp = (long long)blockIdx.x * kWarpsC + wib;
+    if (pf && lp < a.npts) prefetch(lp);
+    int nl = a.nloc && lp < a.npts ? __ldg(a.nloc + lp) : 1;
+
+    for (; lp < a.npts; lp += nw) {
+        float *X = a.x + (size_t)(a.pt0 + lp) * NV * k;
+        const bool zero = nl == 0;
+        const bool more = lp + nw < a.npts;
+        if (a.nloc && more) nl = __ldg(a.nloc + lp + nw);
+        if (pf) {
+            // this point's data (bounded wait; a timeout is never expected: report it, give the
+            // copies a second bounded wait, leave)
+            if (!__all_sync(kAllC, cheb_bar_wait(bar, phase))) {
+                if (lane == 0) atomicOr(a.status, ST_TIMEOUT);
+                cheb_bar_wait(bar, phase);
+                return;
+            }
+            phase ^= 1;
+        } else if (!zero) {
+            const float *src = a.gram + (size_t)lp * k * k;
+            for (int i = 0; i < k; ++i)
+                for (int c = (i & ~31) + lane; c < k; c += 32)
+                    if (c >= i) G[i * SP + c] = __ldg(src + (size_t)i * k + c);
+            for (int e = lane; e < NV * k; e += 32) XS[e] = __ldcg(X + e);
+            for (int e = lane; e < k; e += 32) XS[NV * k + e] = __ldcg(a.cvec + (size_t)lp * k + e);
+            __syncwarp();
+        }
+        if (zero) {
+            if (pf && more) prefetch(lp + nw);
+            // Q = (k-1)/rho I: wbar = 0 and dW = sqrt(rho) I (untouched for rho = 1)
+            if (a.sqrt_infl != 1.0f)
+                for (int r = 0; r < NV; ++r) {
+                    float v[KM / 32], s = 0.0f;
+#pragma unroll
+                    for (int q = 0; q < KM / 32; ++q) {
+                        const int c = lane + 32 * q;
+                        v[q] = c < k ? __ldcg(X + r * k + c) : 0.0f;
+                        s += v[q];
+                    }
+                    const float xb = warp_sum(s) / (float)k;
+#pragma unroll
+                    for (int q = 0; q < KM / 32; ++q) {
+                        const int c = lane + 32 * q;
+                        if (c < k) X[r * k + c] = fmaf(a.sqrt_infl, v[q] - xb, xb);
+                    }
+                }
+            continue;
+        }
+        // ---- A, symmetric, from the staged upper triangle: column c takes A[i][c] for i <= c down
+        // its column (two columns per load) and A[c][i] for i > c along its own row
+        float2 A[NC][S::RH / 2];
+        float f2 = 0.0f, gm = 0.0f;
+#pragma unroll
+        for (int q = 0; q < NC; q += 2) {
+            const int c = cj + 16 * q;
+            float s0 = 0.0f, s1 = 0.0f;
+#pragma unroll
+            for (int g = 0; g < S::RH / 4; ++g) {
+                float v0[4] = {0.0f, 0.0f, 0.0f, 0.0f}, v1[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                if (g < ng) {
+                    const int i0 = row0 + 4 * g;
+                    float4 r0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), r1 = r0;
+                    if (i0 + 3 > c) {
+                        r0 = *reinterpret_cast<const float4 *>(G + c * SP + i0);
+                        r1 = *reinterpret_cast<const float4 *>(G + (c + 1) * SP + i0);
+                    }
+                    const float t0[4] = {r0.x, r0.y, r0.z, r0.w}, t1[4] = {r1.x, r1.y, r1.z, r1.w};
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        float2 up = make_float2(0.0f, 0.0f);
+                        if (i0 + u <= c + 1)
+                            up = *reinterpret_cast<const float2 *>(G + (i0 + u) * SP + c);
+                        v0[u] = i0 + u <= c ? up.x : t0[u];
+                        v1[u] = i0 + u <= c + 1 ? up.y : t1[u];
+                        s0 += fabsf(v0[u]);
+                        s1 += fabsf(v1[u]);
+                        f2 = fmaf(v0[u], v0[u], fmaf(v1[u], v1[u], f2));
+                    }
+                }
+                A[q][2 * g] = make_float2(v0[0], v0[1]);
+                A[q][2 * g + 1] = make_float2(v0[2], v0[3]);
+                A[q + 1][2 * g] = make_float2(v1[0], v1[1]);
+                A[q + 1][2 * g + 1] = make_float2(v1[2], v1[3]);
+            }
+            s0 += __shfl_xor_sync(kAllC, s0, 16);
+            s1 += __shfl_xor_sync(kAllC, s1, 16);
+            gm = fmaxf(gm, fmaxf(s0, s1));
+        }
+        float dg = 0.0f;
+#pragma unroll
+        for (int q = 0; q < KM / 32; ++q) dg += G[(lane + 32 * q) * (SP + 1)];
+        // rows 5..9 of [x; c] in registers, rows 0..4 put aside: the stage is free again
+        float R[5][HC];
+#pragma unroll
+        for (int r = 0; r < 5; ++r)
+#pragma unroll
+            for (int q = 0; q < HC; ++q) {
+                R[r][q] = col + q < k ? XS[(5 + r) * k + col + q] : 0.0f;
+                RS[r * KM + col + q] = col + q < k ? XS[r * k + col + q] : 0.0f;
+            }
+        if (pf) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (pf && more) prefetch(lp + nw);
+        // ---- kappa >= 1 + lambda_max(A) / d from min(Gershgorin, Frobenius, trace)
+        gm = warp_max_c(gm);
+        f2 = warp_sum(f2);
+        dg = warp_sum(dg);
+        const float e = fmaxf(fminf(gm, fminf(sqrtf(f2), dg)), 0.0f);
+        const float kap = fmaf(e * inv_d, 1.0001f, 1.000001f);   // rounding margin
+        int set = 0;
+        while (set <= max_set && !(kap <= ct.kappa_max[set])) ++set;
+        if (set > max_set) {   // beyond the sets in use (or not finite): the rational schedule
+            if (lane == 0) sp.pre_list[atomicAdd(sp.pre_count, 1)] = (int)lp;
+            ++n_hand;
+            continue;
+        }
+        const int n = ct.n[set], co = ct.off[set];
+        const float gam = 2.0f / (d * (ct.kappa_max[set] - 1.0f));
+        bool bad = false;
+#pragma unroll 1
+        for (int pass = 1; pass >= 0; --pass) {   // rows 5..9 (with c), then 0..4
+            if (pass == 0)
+#pragma unroll
+                for (int r = 0; r < 5; ++r)
+#pragma unroll
+                    for (int q = 0; q < HC; ++q) R[r][q] = RS[r * KM + col + q];
+            // ---- R = [dX; c^T]: the rows less their means
+            float mean[5];
+#pragma unroll
+            for (int r = 0; r < 5; ++r) {
+                float s = R[r][0];
+#pragma unroll
+                for (int q = 1; q < HC; ++q) s += R[r][q];
+                mean[r] = warp_sum(s) / (float)k;
+                if (r == 4 && pass) mean[r] = 0.0f;
+#pragma unroll
+                for (int q = 0; q < HC; ++q) R[r][q] = col + q < k ? R[r][q] - mean[r] : 0.0f;
+            }
+            // ---- Clenshaw: b_n = c_n R, b_j = c_j R + 2 b_{j+1} Z - b_{j+2}, result
+            // c_0 R + b_1 Z - b_2, with b_{j+1} Z = gamma b_{j+1} A - b_{j+1}.  Bc holds b_{j+1}
+            // (also in B for the products), Bp b_{j+2}.
+            float Bc[5][HC], Bp[5][HC];
+            auto publish = [&]() {
+#pragma unroll
+                for (int r = 0; r < 5; ++r) {
+                    if constexpr (HC == 2)
+                        *reinterpret_cast<float2 *>(B + r * KM + col) = make_float2(Bc[r][0], Bc[r][1]);
+                    else
+                        B[r * KM + col] = Bc[r][0];
+                }
+                __syncwarp();
+            };
+            {
+                const float2 cn = ct.c[co + n];
+#pragma unroll
+                for (int r = 0; r < 5; ++r)
+#pragma unroll
+                    for (int q = 0; q < HC; ++q) {
+                        Bc[r][q] = (r == 4 && pass ? cn.y : cn.x) * R[r][q];
+                        Bp[r][q] = 0.0f;
+                    }
+            }
+            __syncwarp();
+            publish();
+            for (int j = n - 1; j >= 0; --j) {
+                const float2 cc = ct.c[co + j];
+                float v[5][HC];
+                cheb_product<KM>(B + row0, A, ng, half, v);
+                const float two = j > 0 ? 2.0f : 1.0f;
+#pragma unroll
+                for (int r = 0; r < 5; ++r)
+#pragma unroll
+                    for (int q = 0; q < HC; ++q) {
+                        const float cr = r == 4 && pass ? cc.y : cc.x;
+                        const float z = fmaf(gam, v[r][q], -Bc[r][q]);
+                        const float nb = fmaf(cr, R[r][q], fmaf(two, z, -Bp[r][q]));
+                        Bp[r][q] = Bc[r][q];
+                        Bc[r][q] = nb;
+                    }
+                __syncwarp();   // B is read
+                if (j > 0) publish();
+            }
+            // ---- u = Q^-1 c = S^-1 c / d; X^a_r = xbar_r + dX_r . u + sqrt(k-1) d^-1/2 (dX S^-1/2)_r
+            float u[HC];
+#pragma unroll
+            for (int q = 0; q < HC; ++q) {
+                if (pass) U[col + q] = u[q] = Bc[4][q] * inv_d;
+                else u[q] = U[col + q];
+            }
+#pragma unroll
+            for (int r = 0; r < 5; ++r) {
+                if (r == 4 && pass) break;
+                float s = R[r][0] * u[0];
+#pragma unroll
+                for (int q = 1; q < HC; ++q) s = fmaf(R[r][q], u[q], s);
+                const float base = mean[r] + warp_sum(s);
+#pragma unroll
+                for (int q = 0; q < HC; ++q)
+                    if (col + q < k) {
+                        const float x = fmaf(sc, Bc[r][q], base);
+                        bad |= !isfinite(x);
+                        X[(5 * pass + r) * k + col + q] = x;
+                    }
+            }
+        }
+        if (__any_sync(kAllC, bad) && lane == 0) atomicOr(a.status, ST_NONFINITE);
+        ++n_pts;
+        n_prod += (unsigned long long)n;
+    }
+    if (a.work && lane == 0 && (n_pts | n_hand)) {
+        atomicAdd(a.work, n_pts);
+        atomicAdd(a.work + 1, n_prod);
+        atomicAdd(a.work + 2, n_hand);
+    }
 }
 
 // Five rows of R times NG groups of four rows of A (the loads of later groups run ahead of the
 // multiply-adds: a run-time bound on the groups kept every group waiting for its own loads).
-template <int KM, int NG>
-__device__ __forceinline__ void cheb_product_ng(const float *b,
-                                                const float2 (&A)[ChebShape<KM>::NC][16],
-                                                float (&out)[5][ChebShape<KM>::NC]) {
-    constexpr int NC = ChebShape<KM>::NC;
+template <int NG>
+__device__ __forceinline__ void cheb_block_product_ng(const float *b,
+                                                const float2 (&A)[ChebBlock::NC][16],
+                                                float (&out)[5][ChebBlock::NC]) {
+    constexpr int NC = ChebBlock::NC, KM = ChebBlock::KM;
     const float4 *B4 = reinterpret_cast<const float4 *>(b);
     float2 acc[5][NC];
 #pragma unroll
@@ -244,33 +576,27 @@ __device__ __forceinline__ void cheb_product_ng(const float *b,
 }
 
 // ng groups of the warp's 8 (rows of A beyond them are zero)
-template <int KM>
-__device__ __forceinline__ void cheb_product(const float *b,
-                                             const float2 (&A)[ChebShape<KM>::NC][16], int ng,
-                                             float (&out)[5][ChebShape<KM>::NC]) {
-    if (ng > 6) cheb_product_ng<KM, 8>(b, A, out);
-    else if (ng > 4) cheb_product_ng<KM, 6>(b, A, out);
-    else cheb_product_ng<KM, 4>(b, A, out);
+__device__ __forceinline__ void cheb_block_product(const float *b,
+                                             const float2 (&A)[ChebBlock::NC][16], int ng,
+                                             float (&out)[5][ChebBlock::NC]) {
+    if (ng > 6) cheb_block_product_ng<8>(b, A, out);
+    else if (ng > 4) cheb_block_product_ng<6>(b, A, out);
+    else cheb_block_product_ng<4>(b, A, out);
 }
 
-// What bounds it: per product and point 10 k^2 multiply-adds on the FP32 pipe against 5 k^2 / 2
-// 16-byte broadcasts per 20 k^2 / 4 packed instructions; between products the latency of two
-// barriers and of the exchange, covered by the other points of the SM.  At k <= 64 the phase
-// against A as rows of the block's lanes, re-read from shared memory: 256 x 256, k = 32, 5.8
-// products a point 0.436 -> 0.378 ms; 250 x 187, k = 40, 20.7 products 2.46 -> 2.01 ms; 301 x 215,
-// k = 24, 9.7 products 0.583 -> 0.436 ms; k = 64 the same (256 x 256, 28.4 products 4.28 -> 4.23
-// ms).  192 x 160, k = 128, clustered network, 13.4 products: 77.1 -> 3.44 ms against the split
-// eigensolve, which served k > 64 alone.
-template <int KM>
-__global__ void __launch_bounds__(32 * ChebShape<KM>::NW * ChebShape<KM>::PPB, ChebShape<KM>::MINB)
-    eig_cheb_kernel(EigArgs a, EigSplit sp, const __grid_constant__ ChebTable ct, int max_set) {
-    using S = ChebShape<KM>;
-    constexpr int NW = S::NW, CS = S::CS, NC = S::NC, NE = S::NE, SP = S::SP;
+// k <= 128.  What bounds it: per product and point 10 k^2 multiply-adds on the FP32 pipe; between
+// products the latency of two barriers and of the exchange, covered by the SM's other point.
+// 192 x 160, k = 128, clustered network (13 products a point): 77.1 -> 3.4 ms against the split
+// eigensolve that served k > 64 alone.
+__global__ void __launch_bounds__(32 * ChebBlock::NW, 2)
+    eig_cheb_block_kernel(EigArgs a, EigSplit sp, const __grid_constant__ ChebTable ct,
+                          int max_set) {
+    using S = ChebBlock;
+    constexpr int KM = S::KM, NW = S::NW, CS = S::CS, NC = S::NC, NE = S::NE, SP = S::SP;
     extern __shared__ float4 smem_c4[];
-    __shared__ __align__(8) uint64_t pbar[S::PPB];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int pb = NW == 1 ? wib : 0, w = NW == 1 ? 0 : wib;   // point of the block, its warp
-    float *ws = reinterpret_cast<float *>(smem_c4) + (size_t)pb * S::floats;
+    __shared__ __align__(8) uint64_t pbar;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    float *ws = reinterpret_cast<float *>(smem_c4);
     float *G = ws, *XS = ws + S::off_x, *B = ws + S::off_b, *P = ws + S::off_p, *RD = ws + S::off_r;
     const int k = a.k;
     const float d = a.diag, inv_d = 1.0f / a.diag;
@@ -279,13 +605,13 @@ __global__ void __launch_bounds__(32 * ChebShape<KM>::NW * ChebShape<KM>::PPB, C
     const int rpb = ((k + S::RB - 1) / S::RB + 3) & ~3;       // rows of a block, in groups of 4
     const int row0 = rb * rpb, ng = max(0, min(k - row0, rpb) + 3) / 4;
     unsigned long long n_pts = 0, n_prod = 0, n_hand = 0;
-    const long long stride = (long long)gridDim.x * S::PPB;
+    const long long stride = (long long)gridDim.x;
     // Where the Gram slot's rows are 16-byte multiples (k a multiple of 4) the next point's upper
     // triangle (bulk copies of every row from its first multiple of 4), forecast block and c are
     // fetched into the stage while this point is worked on, counted in bytes on an mbarrier;
     // otherwise the warps load them when the point begins.
     const bool pf = (k & 3) == 0;
-    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&pbar[pb]);
+    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&pbar);
     uint32_t phase = 0;
     auto bulk = [&](float *dst, const float *src, int n) {
         asm volatile(
@@ -314,8 +640,8 @@ __global__ void __launch_bounds__(32 * ChebShape<KM>::NW * ChebShape<KM>::PPB, C
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    point_sync<NW>();
-    long long lp = (long long)blockIdx.x * S::PPB + pb;
+    __syncthreads();
+    long long lp = blockIdx.x;
     if (pf && w == 0 && lp < a.npts) prefetch(lp);
     int nl = a.nloc && lp < a.npts ? __ldg(a.nloc + lp) : 1;
 
@@ -327,10 +653,7 @@ __global__ void __launch_bounds__(32 * ChebShape<KM>::NW * ChebShape<KM>::PPB, C
         if (pf) {
             // this point's data (bounded wait; a timeout is never expected: report it, give the
             // copies a second bounded wait, leave)
-            bool ok = cheb_bar_wait(bar, phase);
-            if constexpr (NW == 1) ok = __all_sync(kAllC, ok);
-            else ok = __syncthreads_and(ok);
-            if (!ok) {
+            if (!__syncthreads_and(cheb_bar_wait(bar, phase))) {
                 if (lane == 0 && w == 0) atomicOr(a.status, ST_TIMEOUT);
                 cheb_bar_wait(bar, phase);
                 return;
@@ -344,7 +667,7 @@ __global__ void __launch_bounds__(32 * ChebShape<KM>::NW * ChebShape<KM>::PPB, C
             for (int e = lane + 32 * w; e < NV * k; e += 32 * NW) XS[e] = __ldcg(X + e);
             for (int e = lane + 32 * w; e < k; e += 32 * NW)
                 XS[NV * k + e] = __ldcg(a.cvec + (size_t)lp * k + e);
-            point_sync<NW>();
+            __syncthreads();
         }
         if (zero) {
             if (pf && w == 0 && more) prefetch(lp + stride);
@@ -369,14 +692,14 @@ __global__ void __launch_bounds__(32 * ChebShape<KM>::NW * ChebShape<KM>::PPB, C
         }
         // ---- A, symmetric, from the staged upper triangle: column c takes A[i][c] for i <= c down
         // its column and A[c][i] for i > c along its own row
-        float2 A[NC][16];   // RR / 2
+        float2 A[NC][16];
         float csum[NC], f2 = 0.0f, dg = 0.0f;
 #pragma unroll
         for (int q = 0; q < NC; ++q) {
             const int c = 32 * (NC * cg + q) + lane;
             csum[q] = 0.0f;
 #pragma unroll
-            for (int g = 0; g < S::RR / 4; ++g) {
+            for (int g = 0; g < 8; ++g) {
                 float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
                 if (g < ng) {
                     const int i0 = row0 + 4 * g;
@@ -418,7 +741,7 @@ __global__ void __launch_bounds__(32 * ChebShape<KM>::NW * ChebShape<KM>::PPB, C
             if (lane == 0) sums[NE * w + t] = v;
         }
         if (pf) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        point_sync<NW>();   // the stage is read: the next point's copies may land in it
+        __syncthreads();   // the stage is read: the next point's copies may land in it
         if (pf && w == 0 && more) prefetch(lp + stride);
         // ---- kappa >= 1 + lambda_max(A) / d from min(Gershgorin, Frobenius, trace)
         float gm = 0.0f;
@@ -444,7 +767,7 @@ __global__ void __launch_bounds__(32 * ChebShape<KM>::NW * ChebShape<KM>::PPB, C
             // beyond the sets in use (or not finite): the next schedule
             if (lane == 0 && w == 0) sp.pre_list[atomicAdd(sp.pre_count, 1)] = (int)lp;
             ++n_hand;
-            point_sync<NW>();   // P and RD are read before the next point writes them
+            __syncthreads();   // P and RD are read before the next point writes them
             continue;
         }
         // ---- R = [dX; c^T]: the nine rows less their means
@@ -454,14 +777,12 @@ __global__ void __launch_bounds__(32 * ChebShape<KM>::NW * ChebShape<KM>::PPB, C
             for (int q = 0; q < CS; ++q) v += sums[row * CS + q];
             return row < NV ? v / (float)k : 0.0f;
         };
-        // (kept where another warp may already be writing the next point's sums at the end)
-        constexpr bool kKeep = NW > 2;
-        float mean[kKeep ? NE : 1];
+        float mean[NE];   // (another warp may be writing the next point's sums at the end)
 #pragma unroll
         for (int t = 0; t < NE; ++t) {
             const int s = NE * w + t, row = s / CS, col = 32 * (s % CS) + lane;
             const float m = row_mean(row);
-            if (kKeep) mean[t] = m;
+            mean[t] = m;
             R[t] = col < k ? R[t] - m : 0.0f;
         }
         // ---- Clenshaw: b_n = c_n R, b_j = c_j R + 2 b_{j+1} Z - b_{j+2}, result
@@ -480,56 +801,29 @@ __global__ void __launch_bounds__(32 * ChebShape<KM>::NW * ChebShape<KM>::PPB, C
                 B[32 * s + lane] = Bc[t];
             }
         }
-        point_sync<NW>();
+        __syncthreads();
         // rows r0 .. r0 + 4 of B times this warp's rows and columns of A
         auto product = [&](int r0, float (&out)[5][NC]) {
-            cheb_product<KM>(B + r0 * KM + row0, A, ng, out);
+            cheb_block_product(B + r0 * KM + row0, A, ng, out);
         };
         for (int j = n - 1; j >= 0; --j) {
             const float2 cj = ct.c[co + j];
             float v[NE];
-            if constexpr (S::RB == 1) {          // one warp: both passes are its own
 #pragma unroll
-                for (int p = 0; p < 2; ++p) {
-                    float o[5][NC];
-                    product(5 * p, o);
-#pragma unroll
-                    for (int rr = 0; rr < 5; ++rr) v[5 * p + rr] = o[rr][0];
-                }
-                __syncwarp();
-            } else if constexpr (S::RB == 2) {   // the other warp's rows first, then its own
+            for (int p = 0; p < 2; ++p) {
                 float o[5][NC];
-                product(5 * (1 - w), o);
-                float *pw = P + 5 * (1 - w) * KM + lane;
+                product(5 * p, o);
+                float *pw = P + (rb * kRowsC + 5 * p) * KM + 32 * NC * cg + lane;
 #pragma unroll
                 for (int rr = 0; rr < 5; ++rr)
 #pragma unroll
                     for (int q = 0; q < NC; ++q) pw[rr * KM + 32 * q] = o[rr][q];
-                product(5 * w, o);
-                point_sync<NW>();
-                const float *pr = P + 5 * w * KM + lane;
+            }
+            __syncthreads();
 #pragma unroll
-                for (int rr = 0; rr < 5; ++rr)
-#pragma unroll
-                    for (int q = 0; q < NC; ++q)
-                        v[2 * rr + q] = o[rr][q] + pr[rr * KM + 32 * q];
-            } else {                             // every row block's sums through shared memory
-#pragma unroll
-                for (int p = 0; p < 2; ++p) {
-                    float o[5][NC];
-                    product(5 * p, o);
-                    float *pw = P + (rb * kRowsC + 5 * p) * KM + 32 * NC * cg + lane;
-#pragma unroll
-                    for (int rr = 0; rr < 5; ++rr)
-#pragma unroll
-                        for (int q = 0; q < NC; ++q) pw[rr * KM + 32 * q] = o[rr][q];
-                }
-                point_sync<NW>();
-#pragma unroll
-                for (int t = 0; t < NE; ++t) {
-                    const float *pr = P + 32 * (NE * w + t) + lane;
-                    v[t] = (pr[0] + pr[kRowsC * KM]) + (pr[2 * kRowsC * KM] + pr[3 * kRowsC * KM]);
-                }
+            for (int t = 0; t < NE; ++t) {
+                const float *pr = P + 32 * (NE * w + t) + lane;
+                v[t] = (pr[0] + pr[kRowsC * KM]) + (pr[2 * kRowsC * KM] + pr[3 * kRowsC * KM]);
             }
 #pragma unroll
             for (int t = 0; t < NE; ++t) {
@@ -542,7 +836,7 @@ __global__ void __launch_bounds__(32 * ChebShape<KM>::NW * ChebShape<KM>::PPB, C
                 Bc[t] = nb;
                 B[32 * s + lane] = nb;
             }
-            point_sync<NW>();
+            __syncthreads();
         }
         // ---- u = Q^-1 c = S^-1 c / d; X^a_r = xbar_r + dX_r . u + sqrt(k-1) d^-1/2 (dX S^-1/2)_r
 #pragma unroll
@@ -552,12 +846,12 @@ __global__ void __launch_bounds__(32 * ChebShape<KM>::NW * ChebShape<KM>::PPB, C
             const float v = warp_sum(R[t] * u);
             if (lane == 0) dots[s] = v;
         }
-        point_sync<NW>();
+        __syncthreads();
         bool bad = false;
 #pragma unroll
         for (int t = 0; t < NE; ++t) {
             const int s = NE * w + t, row = s / CS, col = 32 * (s % CS) + lane;
-            float v = kKeep ? mean[kKeep ? t : 0] : row_mean(row);
+            float v = mean[t];
 #pragma unroll
             for (int q = 0; q < CS; ++q) v += dots[row * CS + q];
             if (row < NV && col < k) {
@@ -577,24 +871,21 @@ __global__ void __launch_bounds__(32 * ChebShape<KM>::NW * ChebShape<KM>::PPB, C
     }
 }
 
+constexpr size_t kBlockSmem = (size_t)ChebBlock::floats * sizeof(float);
 template <int KM>
 constexpr size_t cheb_smem() {
-    return (size_t)ChebShape<KM>::floats * ChebShape<KM>::PPB * sizeof(float);
+    return (size_t)ChebShape<KM>::floats * kWarpsC * sizeof(float);
 }
 
-template <int KM>
-cudaError_t cheb_prepare_km(int k, int *grid) {
-    using S = ChebShape<KM>;
-    const size_t smem = cheb_smem<KM>();
-    cudaError_t e = cudaFuncSetAttribute(eig_cheb_kernel<KM>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t cheb_prepare(const void *kern, int threads, size_t smem, int k, int *grid) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, eig_cheb_kernel<KM>,
-                                                      32 * S::NW * S::PPB, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     *grid = sms * per_sm;
@@ -604,10 +895,9 @@ cudaError_t cheb_prepare_km(int k, int *grid) {
 
 template <int KM>
 cudaError_t cheb_launch_km(const EigArgs &a, const EigSplit &sp, int grid, cudaStream_t s) {
-    using S = ChebShape<KM>;
-    const long long need = ((long long)a.npts + S::PPB - 1) / S::PPB;
+    const long long need = ((long long)a.npts + kWarpsC - 1) / kWarpsC;
     const unsigned blocks = (unsigned)(need < grid ? need : grid);
-    eig_cheb_kernel<KM><<<blocks, 32 * S::NW * S::PPB, cheb_smem<KM>(), s>>>(
+    eig_cheb_kernel<KM><<<blocks, 32 * kWarpsC, cheb_smem<KM>(), s>>>(
         a, sp, cheb_table(a.k), cheb_max_set(a.k));
     return cudaGetLastError();
 }
@@ -615,9 +905,13 @@ cudaError_t cheb_launch_km(const EigArgs &a, const EigSplit &sp, int grid, cudaS
 }  // namespace
 
 cudaError_t eigen_cheb_prepare(int k, int *grid) {
-    if (k <= 32) return cheb_prepare_km<32>(k, grid);
-    if (k <= 64) return cheb_prepare_km<64>(k, grid);
-    if (k <= kChebSplitMaxK) return cheb_prepare_km<128>(k, grid);
+    if (k <= 32)
+        return cheb_prepare((const void *)eig_cheb_kernel<32>, 32 * kWarpsC, cheb_smem<32>(), k, grid);
+    if (k <= 64)
+        return cheb_prepare((const void *)eig_cheb_kernel<64>, 32 * kWarpsC, cheb_smem<64>(), k, grid);
+    if (k <= kChebSplitMaxK)
+        return cheb_prepare((const void *)eig_cheb_block_kernel, 32 * ChebBlock::NW, kBlockSmem, k,
+                            grid);
     return cudaErrorInvalidValue;
 }
 
@@ -627,7 +921,12 @@ cudaError_t launch_eigen_cheb_transform(const EigArgs &a, const EigSplit &sp, in
     if (!sp.pre_list || !sp.pre_count || grid < 1) return cudaErrorInvalidValue;
     if (a.k <= 32) return cheb_launch_km<32>(a, sp, grid, s);
     if (a.k <= 64) return cheb_launch_km<64>(a, sp, grid, s);
-    if (a.k <= kChebSplitMaxK) return cheb_launch_km<128>(a, sp, grid, s);
+    if (a.k <= kChebSplitMaxK) {
+        const unsigned blocks = (unsigned)(a.npts < grid ? a.npts : grid);
+        eig_cheb_block_kernel<<<blocks, 32 * ChebBlock::NW, kBlockSmem, s>>>(
+            a, sp, cheb_table(a.k), cheb_max_set(a.k));
+        return cudaGetLastError();
+    }
     return cudaErrorInvalidValue;
 }
 
