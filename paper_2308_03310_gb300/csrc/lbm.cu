@@ -10,24 +10,29 @@
 // rest state (exact weights).
 //
 // Up to four steps per launch (lbm_kernel<T>), in registers.  A warp owns a window of 64 columns of
-// one member, two neighbouring ones per lane, and marches along y: per row it loads the nine
-// populations (coalesced, one row ahead), and the T steps run as a pipeline of T stages, stage s
-// one row behind stage s - 1.  A collision's outputs stream to the stage after it: along x with
-// one shuffle per direction and pair, along y by waiting in registers (those with c_y = -1 are
-// used at once, c_y = 0 one row later, c_y = +1 two rows later).  The last stage's populations are
-// streamed the same way and stored, coalesced.  A window loses one column per side and step, so
-// neighbouring windows overlap by the halo, and so do the segments of rows a member is cut into.
-// No shared memory and no barrier: a form that kept four steps' rows in shared memory (36
-// accesses of 8 bytes per pair of nodes and step, four barriers per eight rows) was bound by
-// them, at 1.26 to 1.45 ms per four steps of 1024^2, k = 64, whatever the tile.
+// one member, two neighbouring ones per lane, and marches along y; the T steps run as a pipeline of
+// T stages, stage s one row behind stage s - 1.  A collision's outputs stream to the stage after it:
+// along x with one shuffle per direction and pair, along y by waiting in registers (those with
+// c_y = -1 are used at once, c_y = 0 one row later, c_y = +1 two rows later).  The last stage's
+// populations are streamed the same way and stored, coalesced.  A window loses one column per side
+// and step, so neighbouring windows overlap by the halo, and so do the segments of rows a member
+// is cut into.  Rows arrive by asynchronous copies three rows ahead in the warp's own ring in
+// shared memory (nothing spills then, and a warp is never behind the memory's latency), the force
+// in a longer one that every stage reads its row from.  A block is one warp, so that member,
+// strip and row addresses are uniform, and there is no block barrier.  A form that kept four steps'
+// rows in shared memory (36 accesses of 8 bytes per pair of nodes and step, four barriers per
+// eight rows) was bound by them, at 1.26 to 1.45 ms per four steps of 1024^2, k = 64.
 //
-// Measured (four steps, with a force; before: two launches of two steps through shared memory
-// with the collision written as g + omega (g_eq - g) per direction):
-//   1024^2, k = 64: 1759 -> 1031 us (64 % of the copy rate in its own 4.8 GB);
-//   256^2, k = 32: 71.1 -> 42.1 us; 509 x 380, k = 20: 185 -> 74.5 us; 64^2, k = 20: 8.6 -> 8.3 us.
-// Bound: the FP32 pipe (53 % active at 256^2, k = 64) behind the latency of three warps per
-// scheduler, which is what 168 registers allow; 128 registers (four warps) spill and measured
-// 1337 us, the row loop without its unrolling by two (moves between the waiting rows) 1148 us.
+// Measured, four steps with a force: two launches of two steps through shared memory, the
+// collision written as g + omega (g_eq - g) per direction -> this pipeline with the next row in
+// registers -> with the ring:
+//   1024^2, k = 64: 1759 -> 1031 -> 852 us (84 % of the copy rate in its own 4.8 GB);
+//   256^2, k = 32: 71.1 -> 42.2 -> 39.1 us; 509 x 380, k = 20: 185 -> 74.5 -> 74.9 us;
+//   64^2, k = 20: 8.6 -> 8.2 -> 7.4 us; 250 x 187, k = 40 (no force): 36.4 -> 34.8 us.
+// Rings of two rows 962 us, two warps a block 865 us.  The row loop unrolled by four gains 1 to 6 %
+// more from 128 x 128 on (847 us at 1024^2) but makes a 32^2 cycle, where fetching the code counts,
+// 6 % slower.  Bound: memory at 1024^2; the FP32 pipe
+// and the latency of three warps per scheduler (what 168 registers allow) at smaller grids.
 #include <math.h>
 
 #include "common.cuh"
@@ -38,8 +43,7 @@ namespace {
 
 // The collision works on two nodes at once: every quantity is a float2 (node pair) and every
 // operation a packed FP32 instruction, which rounds each lane exactly as the scalar operation
-// would.  Both kernels use this function (the single-step kernel with a node in both lanes),
-// so their arithmetic is the same.
+// would.
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
@@ -137,8 +141,12 @@ __device__ __forceinline__ void collide2(const float2 (&g)[NV], float2 fx, float
 }
 
 constexpr int kWin = 64;                      // columns of a warp's window
-constexpr int kLbmWarps = 4;                  // warps (windows) per CTA
-constexpr int kLbmBlocks = 3;                 // CTAs per SM
+constexpr int kLbmBlocks = 12;                // CTAs, of one warp, per SM
+// rows of the staging ring (one less in flight), and of the force's, which the stages read up to
+// T - 1 rows back (launches of one or two steps keep more warps per SM: with four rows a launch of
+// one step takes 1075 us at 1024^2, k = 64, with two 820)
+constexpr int lbm_ahead(int T) { return T > 2 ? 4 : 2; }
+constexpr int lbm_force_ring(int T) { return T > 2 ? 8 : T > 1 ? 4 : 2; }
 // halo columns on either side of a strip: T, rounded up to whole pairs
 constexpr int lbm_halo(int T) { return (T + 1) & ~1; }
 constexpr int lbm_strip(int T) { return kWin - 2 * lbm_halo(T); }
@@ -178,17 +186,32 @@ __device__ __forceinline__ void stream_y(const float2 (&s)[NV], Waiting &w, floa
     }
 }
 
+// Asynchronous copies of a lane's own 4, 8 or 16 bytes into its slot of the staging ring.
+__device__ __forceinline__ void async4(void *d, const void *s) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(d)), "l"(s) : "memory");
+}
+__device__ __forceinline__ void async8(void *d, const void *s) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(d)), "l"(s) : "memory");
+}
+__device__ __forceinline__ void async16(void *d, const void *s) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(d)), "l"(s) : "memory");
+}
+
 // T steps.  Unit u: strip (fastest), segment of H rows, member.  kEven: nx is even, so a window's
 // pairs are 8-byte aligned and never split by the periodic wrap.
 template <int T, bool kForce, bool kEven>
-__global__ void __launch_bounds__(32 * kLbmWarps, kLbmBlocks)
+__global__ void __launch_bounds__(32, kLbmBlocks)
     lbm_kernel(const float *__restrict__ gin, float *__restrict__ gout,
                const float2 *__restrict__ force, int nx, int ny, int H, int strips, int segs,
-               long long units, LbmCoef coef) {
+               LbmCoef coef) {
     constexpr int HX = lbm_halo(T), TX = lbm_strip(T);
-    const long long u = (long long)blockIdx.x * kLbmWarps + (threadIdx.x >> 5);
-    if (u >= units) return;
-    const int c = threadIdx.x & 31;
+    constexpr int kAhead = lbm_ahead(T), kForceRing = lbm_force_ring(T);
+    static_assert(kForceRing >= kAhead + T - 1, "a stage's row of the force is still there");
+    const unsigned u = blockIdx.x;
+    const int c = threadIdx.x;
     const int strip = (int)(u % strips), seg = (int)(u / strips % segs);
     const size_t npts = (size_t)nx * ny;
     const size_t mbase = (size_t)(u / strips / segs) * NV * npts;
@@ -198,25 +221,35 @@ __global__ void __launch_bounds__(32 * kLbmWarps, kLbmBlocks)
     // row l of the segment is y = ys - T + l (periodic), l < rows
     const int rows = ye - ys + 2 * T;
     int y = posmod(ys - T, ny);              // of the row to be loaded next
-    auto load = [&](float2 (&g)[NV], float2 &f0, float2 &f1) {
-        const size_t p = (size_t)y * nx;
+    // a lane reads only what it copied itself: no exchange, no barrier
+    __shared__ float2 ring[kAhead][NV][32];
+    __shared__ float4 fring[kForce ? kForceRing : 1][32];
+    auto load = [&](int l) {                 // row l into its slot; a group even when there is none
+        if (l < rows) {
+            const size_t p = (size_t)y * nx;
 #pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            const float *a = src + (size_t)q * npts + p;
-            g[q] = kEven ? __ldcs(reinterpret_cast<const float2 *>(a + xa))
-                         : make_float2(__ldcs(a + xa), __ldcs(a + xb));
-        }
-        if (kForce) {
-            if (kEven) {                     // the pair's force: one 16-byte load
-                const float4 f = __ldg(reinterpret_cast<const float4 *>(force + p + xa));
-                f0 = make_float2(f.x, f.y);
-                f1 = make_float2(f.z, f.w);
-            } else {
-                f0 = __ldg(force + p + xa);
-                f1 = __ldg(force + p + xb);
+            for (int q = 0; q < NV; ++q) {
+                const float *a = src + (size_t)q * npts + p;
+                float2 *d = ring[l & (kAhead - 1)][q];
+                if (kEven) {
+                    async8(d + c, a + xa);
+                } else {
+                    async4(&d[c].x, a + xa);
+                    async4(&d[c].y, a + xb);
+                }
             }
+            if (kForce) {
+                float4 *f = fring[l & (kForceRing - 1)];
+                if (kEven) {                 // the pair's force: one 16-byte copy
+                    async16(f + c, force + p + xa);
+                } else {
+                    async8(&f[c].x, force + p + xa);
+                    async8(&f[c].z, force + p + xb);
+                }
+            }
+            y = y + 1 == ny ? 0 : y + 1;
         }
-        y = y + 1 == ny ? 0 : y + 1;
+        asm volatile("cp.async.commit_group;" ::: "memory");
     };
     // targets: columns x0 + t, x0 + t + 1 of the strip and grid (for an even nx both or neither)
     const int t = 2 * c - HX;
@@ -228,27 +261,27 @@ __global__ void __launch_bounds__(32 * kLbmWarps, kLbmBlocks)
     for (int i = 0; i < (T > 1 ? T - 1 : 1); ++i)
 #pragma unroll
         for (int k = 0; k < 3; ++k) w[i].zero[k] = w[i].up1[k] = w[i].up2[k] = make_float2(0.0f, 0.0f);
-    float2 fx[T], fy[T];                     // the force of the stages' rows
+    if (kForce)                              // the rows before the first: any finite force
 #pragma unroll
-    for (int i = 0; i < T; ++i) fx[i] = fy[i] = make_float2(0.0f, 0.0f);
-    float2 nxt[NV], nf0 = fx[0], nf1 = fx[0];
-    load(nxt, nf0, nf1);
+        for (int r = 0; r < kForceRing; ++r) fring[r][c] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+    for (int r = 0; r < kAhead - 1; ++r) load(r);
 #pragma unroll 2
     for (int l = 0; l < rows; ++l) {
         float2 g[NV], o[NV], s[NV];
+        asm volatile("cp.async.wait_group %0;" ::"n"(kAhead - 2) : "memory");
 #pragma unroll
-        for (int q = 0; q < NV; ++q) g[q] = nxt[q];
-#pragma unroll
-        for (int i = T - 1; i > 0; --i) {
-            fx[i] = fx[i - 1];
-            fy[i] = fy[i - 1];
-        }
-        fx[0] = make_float2(nf0.x, nf1.x);
-        fy[0] = make_float2(nf0.y, nf1.y);
-        if (l + 1 < rows) load(nxt, nf0, nf1);
+        for (int q = 0; q < NV; ++q) g[q] = ring[l & (kAhead - 1)][q][c];
+        load(l + kAhead - 1);
 #pragma unroll
         for (int i = 0; i < T; ++i) {        // stage i + 1, row l - i
-            collide2<kForce>(g, fx[i], fy[i], coef, o);
+            float2 fx = make_float2(0.0f, 0.0f), fy = fx;
+            if (kForce) {
+                const float4 f = fring[(l - i) & (kForceRing - 1)][c];
+                fx = make_float2(f.x, f.z);
+                fy = make_float2(f.y, f.w);
+            }
+            collide2<kForce>(g, fx, fy, coef, o);
             stream_x(o, s);
             if (i + 1 < T) stream_y(s, w[i], g);
         }
@@ -275,7 +308,7 @@ __global__ void __launch_bounds__(32 * kLbmWarps, kLbmBlocks)
 template <int T>
 int segment_rows(int nx, int ny, int nmem, int sms) {
     const long long lines = (long long)((nx + lbm_strip(T) - 1) / lbm_strip(T)) * nmem;
-    constexpr int wmax = kLbmBlocks * kLbmWarps / 4;
+    constexpr int wmax = kLbmBlocks / 4;
     static_assert(wmax == 3, "the units of a row");
     const double unit[wmax] = {0.0, 1.7, 2.4};
     int best = ny;
@@ -297,15 +330,14 @@ template <int T, bool kForce>
 cudaError_t launch_steps(const float *gin, float *gout, const float2 *force, int nx, int ny,
                          int nmem, float tau, cudaStream_t s, int rows) {
     const int strips = (nx + lbm_strip(T) - 1) / lbm_strip(T), segs = (ny + rows - 1) / rows;
-    const long long units = (long long)strips * segs * nmem;
-    const unsigned grid = (unsigned)((units + kLbmWarps - 1) / kLbmWarps);
+    const unsigned units = (unsigned)strips * segs * nmem;   // windows of 56 columns and more
     const LbmCoef coef = lbm_coef(tau);
     if (nx % 2 == 0)
-        lbm_kernel<T, kForce, true><<<grid, 32 * kLbmWarps, 0, s>>>(gin, gout, force, nx, ny, rows,
-                                                                    strips, segs, units, coef);
+        lbm_kernel<T, kForce, true>
+            <<<units, 32, 0, s>>>(gin, gout, force, nx, ny, rows, strips, segs, coef);
     else
-        lbm_kernel<T, kForce, false><<<grid, 32 * kLbmWarps, 0, s>>>(gin, gout, force, nx, ny, rows,
-                                                                     strips, segs, units, coef);
+        lbm_kernel<T, kForce, false>
+            <<<units, 32, 0, s>>>(gin, gout, force, nx, ny, rows, strips, segs, coef);
     return cudaGetLastError();
 }
 

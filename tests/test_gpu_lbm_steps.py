@@ -1,7 +1,7 @@
 """The four-step D2Q9 launch against four single steps, bit for bit: grids whose strips (64 columns)
-and segments (8 rows and more) are ragged, narrower than the halo, or wrap onto themselves, all
-three staging paths (TMA, 16-byte and 4-byte copies), with and without a force, and the rests
-of step counts that are not multiples of four."""
+and segments of rows are ragged, narrower than the halo, or wrap onto themselves, even widths
+(8-byte copies) and odd ones (4-byte), with and without a force, and the rests of step counts
+that are not multiples of four."""
 import numpy as np
 import pytest
 
@@ -39,11 +39,11 @@ def _forecasts(nx, ny, k, forced, steps):
 @pytest.mark.parametrize("forced", [True, False])
 @pytest.mark.parametrize("nx,ny,k", [
     (64, 8, 2),       # one strip, one segment: both edges wrap
-    (256, 64, 3),     # interior strips by TMA
-    (192, 203, 2),    # TMA strips, a ragged last segment
-    (132, 50, 2),     # a last strip of four columns
-    (130, 37, 2),     # 4-byte staging, even width
-    (67, 29, 2),      # 4-byte staging, odd width, a last strip of three columns
+    (256, 64, 3),     # interior strips
+    (192, 203, 2),    # a ragged last segment
+    (132, 50, 2),     # a ragged last strip
+    (130, 37, 2),     # an even width off the multiples of four
+    (67, 29, 2),      # an odd width: 4-byte copies, a ragged last strip
     (20, 12, 2),      # narrower than a strip
     (3, 2, 2),        # narrower than the halo
     (1, 1, 2),
