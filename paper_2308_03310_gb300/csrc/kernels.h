@@ -200,12 +200,11 @@ cudaError_t launch_eigen_rational(const EigArgs &a, const EigSplit &sp, int grid
 // (LETKF_EIG_CHEBYSHEV, k <= kChebMaxK): coefficients of T_j in s = (2t - kappa_max - 1) /
 // (kappa_max - 1), FP32 copies of the FP64 interpolants, the first set that covers a point's
 // condition bound is used.
-constexpr int kChebSets = 15;
-constexpr int kChebMaxDeg = 36;
+constexpr int kChebSets = 20;
 constexpr int kChebMaxK = 64;       // LETKF_EIG_CHEBYSHEV; beyond, up to kChebSplitMaxK, AUTO may
 constexpr int kChebSplitMaxK = 128;  // choose it, with the sets up to kappa 400
-constexpr int kChebBigSets = 23;
-constexpr int kChebCoefs = 1100;
+constexpr int kChebBigSets = 28;
+constexpr int kChebCoefs = 1136;
 struct ChebTable {
     float kappa_max[kChebBigSets];
     int n[kChebBigSets];            // degree
