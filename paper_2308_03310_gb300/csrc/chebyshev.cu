@@ -141,11 +141,12 @@ const ChebTable &cheb_table(int k) {
 
 // The largest set the transform uses for ensemble size k.  k <= 64: degrees up to 9k/16 (at least
 // 4): a product with A costs ~20 k^2 flops, the rational schedule's tridiagonalization and
-// transform ~(4/3) k^3 + 40 k^2 at a lower issue efficiency; at k = 64 the two measured equal
-// near degree 36, and the break-even degree scales with k.  Points beyond go to the rational
-// schedule, so the Chebyshev schedule never costs much more than the rational one.  k > 64: the
-// alternative is the split eigensolve, ~2.5 us a point at k = 128 against ~10 ns a product:
-// every set is used up to degree 1.4 k.
+// transform ~(4/3) k^3 + 40 k^2 at a lower issue efficiency, so the break-even degree scales with
+// k.  The line was drawn where the two measured equal at k = 64 (degree 36) and stays, so that
+// the same points take the same schedule, although products have become cheaper (break-even
+// measured since at 7, 17, 24, 28, 31 and 55 for k = 8, 16, 20, 24, 32 and 40 to 64; a point beyond
+// goes to the rational schedule).  k > 64: the alternative is the split eigensolve, ~2.5 us a
+// point at k = 128 against ~10 ns a product: every set is used up to degree 1.4 k.
 int cheb_max_set(int k) {
     const ChebTable &t = cheb_table(k);
     const int nsets = k <= kChebMaxK ? kChebSets : kChebBigSets;
@@ -221,6 +222,21 @@ __device__ __forceinline__ float warp_max_c(float v) {
     return v;
 }
 
+// Four entries of a row of R.  At KM = 64 the load stays where it is written: moved ahead by the
+// compiler, the loads pushed pointers and counters out of the 255 registers (256 x 256, 28 products
+// 3.76 -> 3.63 ms, 1024 x 1024, three products 11.9 -> 11.2 ms); at KM = 32, with registers to
+// spare, moving them is better (301 x 215, k = 24 0.428 ms pinned, 0.414 not).
+template <int KM>
+__device__ __forceinline__ float4 row4(const float4 *p) {
+    if constexpr (KM == 32) return *p;
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"((uint32_t)__cvta_generic_to_shared(p))
+                 : "memory");
+    return v;
+}
+
 // Five rows of R (b, row stride KM, this half warp's first row of A) times NG groups of four rows of
 // A per half warp; sums over both half warps, each lane keeping half of its columns.  (With a
 // run-time bound on the groups every group waited for its own loads.)
@@ -235,7 +251,7 @@ __device__ __forceinline__ void cheb_product_ng(
     for (int g = 0; g < NG; ++g)
 #pragma unroll
         for (int rr = 0; rr < 5; ++rr) {
-            const float4 v = B4[rr * (KM / 4) + g];
+            const float4 v = row4<KM>(B4 + rr * (KM / 4) + g);
 #pragma unroll
             for (int q = 0; q < NC; ++q)
                 acc[rr][q] = g ? __ffma2_rn(make_float2(v.x, v.y), A[q][2 * g], acc[rr][q])
