@@ -101,9 +101,8 @@ extern "C" {
                                     degree 4 at kappa_max = 1.1 up to 36 at 16) and applied to
                                     [dX; c^T] by Clenshaw's recurrence, one product with A per
                                     degree.  No factorization or tridiagonalization.  Degrees
-                                    up to 9k/16 are used (kappa_max 16 at k = 64, 4 at k = 32),
-                                    about where a product costs as much as the RATIONAL
-                                    schedule; a point beyond is passed to RATIONAL.
+                                    up to 9k/16 are used (kappa_max 16 at k = 64, 4 at k = 32);
+                                    a point beyond is passed to RATIONAL.
                                     Pays where Q is well conditioned (ensemble spread small
                                     against the observation error).  A probe's eigenvalues come
                                     from a tridiagonalization and an eigenvalue-only QL.      */

@@ -53,7 +53,7 @@ def test_four_step_launch_equals_single_steps(nx, ny, k, forced):
     assert np.array_equal(many, single)
 
 
-@pytest.mark.parametrize("steps", [4, 5, 6, 7, 11])
+@pytest.mark.parametrize("steps", [4, 5, 6, 7, 9, 10, 11])
 def test_step_counts_with_rests_equal_single_steps(steps):
     many, single = _forecasts(140, 45, 2, True, steps)
     assert np.array_equal(many, single)
