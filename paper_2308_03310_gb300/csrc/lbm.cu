@@ -63,13 +63,19 @@ __device__ __forceinline__ float2 rcp2(float2 x) {
     return fma2(y, e, y);
 }
 
+// Relaxation times beyond 2: 1 - omega is no FP32 number for omega < 1/2, and rounding it would
+// change omega by up to 3e-8 absolutely (1.3e-5 of it at tau = 1000) with the same sign at every
+// node and step.  The collision then keeps g apart from what it adds to it: out = g + (omega
+// (g_eq - g) + 3 w c.F), nine additions more.
+inline bool slow_relaxation(float tau) { return 1.0f / tau < 0.5f; }
+
 // The collision's constants, from omega = 1 / tau in FP32 (host, FP64).  They satisfy
-// rest + 9 rho = 1 and rest + 12 mom = 1 (rho, mom as two FP32 words each) and quad = 3 quad6
-// exactly, so that a collision conserves mass and momentum up to the rounding of its sums: a
-// constant off by one ulp would act on every node and step with the same sign (an error of
-// 6e-6 after 100 steps, measured, against 5e-7).
+// rest + 9 rho = 1 and rest + 12 mom = 1 (slow relaxation: rest + 9 rho = 0 and rest + 12 mom = 0;
+// rho, mom as two FP32 words each) and quad = 3 quad6 exactly, so that a collision conserves mass
+// and momentum up to the rounding of its sums: a constant off by one ulp would act on every node
+// and step with the same sign (an error of 6e-6 after 100 steps, measured, against 5e-7).
 struct LbmCoef {
-    float rest;             // 1 - omega
+    float rest;             // 1 - omega (exact for omega >= 1/2); slow relaxation: -omega
     float rho, rho_lo;      // omega / 9
     float mom, mom_lo;      // omega / 12
     float nquad6, quad, quad8, quad4;   // -omega / 6, omega / 2, omega / 8, omega / 4
@@ -77,8 +83,8 @@ struct LbmCoef {
 LbmCoef lbm_coef(float tau) {
     LbmCoef c;
     const double omega = (double)(1.0f / tau);
-    c.rest = (float)(1.0 - omega);
-    const double t = 1.0 - (double)c.rest;   // the relaxation in effect (omega for tau <= 2)
+    c.rest = (float)(slow_relaxation(tau) ? -omega : 1.0 - omega);
+    const double t = omega;
     c.rho = (float)(t / 9.0);
     c.rho_lo = (float)(t / 9.0 - (double)c.rho);
     c.mom = (float)(t / 12.0);
@@ -103,8 +109,10 @@ LbmCoef lbm_coef(float tau) {
 //     b / 4 + omega (P + Q) / 8 +- omega R / 4, b = omega (drho / 9 - (P + Q) / 6);
 //   odd: 4 m_x, 4 m_y, m_x +- m_y, m = (omega j + F) / 12.
 // 61 packed operations for two nodes (the form g + omega (g_eq - g) per direction took 95).  Error
-// after 100 steps against 64 bits (tau = 0.52, u = 0.02, emulated): 2.1e-6 -> 5e-7.
-template <bool kForce>
+// after 100 steps against 64 bits (tau = 0.52, u = 0.02, emulated): 2.1e-6 -> 5e-7.  kSlow (the
+// slow relaxation above): -omega g in place of (1 - omega) g, and g added last; error at tau = 30 /
+// 100 / 1000 with 1 - omega rounded 1.5e-6 / 6.1e-7 / 7.7e-7, so 2.5e-7.
+template <bool kForce, bool kSlow>
 __device__ __forceinline__ void collide2(const float2 (&g)[NV], float2 fx, float2 fy,
                                          const LbmCoef &c, float2 (&out)[NV]) {
     const float2 s0 = add2(g[0], g[8]), s1 = add2(g[1], g[7]), s2 = add2(g[2], g[6]),
@@ -138,6 +146,9 @@ __device__ __forceinline__ void collide2(const float2 (&g)[NV], float2 fx, float
     out[1] = fma2(dup2(-4.0f), my, fma2(r, g[1], ay));
     out[5] = fma2(dup2(4.0f), mx, fma2(r, g[5], ax));
     out[3] = fma2(dup2(-4.0f), mx, fma2(r, g[3], ax));
+    if (kSlow)
+#pragma unroll
+        for (int q = 0; q < NV; ++q) out[q] = add2(out[q], g[q]);
 }
 
 constexpr int kWin = 64;                      // columns of a warp's window
@@ -202,7 +213,7 @@ __device__ __forceinline__ void async16(void *d, const void *s) {
 
 // T steps.  Unit u: strip (fastest), segment of H rows, member.  kEven: nx is even, so a window's
 // pairs are 8-byte aligned and never split by the periodic wrap.
-template <int T, bool kForce, bool kEven>
+template <int T, bool kForce, bool kEven, bool kSlow>
 __global__ void __launch_bounds__(32, kLbmBlocks)
     lbm_kernel(const float *__restrict__ gin, float *__restrict__ gout,
                const float2 *__restrict__ force, int nx, int ny, int H, int strips, int segs,
@@ -281,7 +292,7 @@ __global__ void __launch_bounds__(32, kLbmBlocks)
                 fx = make_float2(f.x, f.z);
                 fy = make_float2(f.y, f.w);
             }
-            collide2<kForce>(g, fx, fy, coef, o);
+            collide2<kForce, kSlow>(g, fx, fy, coef, o);
             stream_x(o, s);
             if (i + 1 < T) stream_y(s, w[i], g);
         }
@@ -332,12 +343,11 @@ cudaError_t launch_steps(const float *gin, float *gout, const float2 *force, int
     const int strips = (nx + lbm_strip(T) - 1) / lbm_strip(T), segs = (ny + rows - 1) / rows;
     const unsigned units = (unsigned)strips * segs * nmem;   // windows of 56 columns and more
     const LbmCoef coef = lbm_coef(tau);
-    if (nx % 2 == 0)
-        lbm_kernel<T, kForce, true>
-            <<<units, 32, 0, s>>>(gin, gout, force, nx, ny, rows, strips, segs, coef);
-    else
-        lbm_kernel<T, kForce, false>
-            <<<units, 32, 0, s>>>(gin, gout, force, nx, ny, rows, strips, segs, coef);
+    const bool slow = slow_relaxation(tau);
+    auto *const f = nx % 2 == 0
+        ? (slow ? lbm_kernel<T, kForce, true, true> : lbm_kernel<T, kForce, true, false>)
+        : (slow ? lbm_kernel<T, kForce, false, true> : lbm_kernel<T, kForce, false, false>);
+    f<<<units, 32, 0, s>>>(gin, gout, force, nx, ny, rows, strips, segs, coef);
     return cudaGetLastError();
 }
 
