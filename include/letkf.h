@@ -110,8 +110,9 @@ extern "C" {
 /* FP32 Gram schedules (letkf_config.gram_tile; applies to LETKF_FP32 only, and PIPE / TEAM to
  * k >= 17 only: k <= 16 has one CUDA-core schedule). */
 #define LETKF_GRAM_AUTO   0  /* LETKF_GRAM_TENSOR from 1,024 grid points on, where the network's
-                                products fit its buffer (n_obs x k (k + 3) / 2 entries of 6
-                                bytes within 2 GiB) and coordinates and cutoff are below 65536
+                                products (n_obs x k (k + 3) / 2 entries of 6 bytes) fit in 2
+                                GiB and in letkf_config.chunk_bytes, eight grid rows (or the
+                                grid) in a chunk, and coordinates and cutoff are below 65536
                                 and 2896 cells.  Otherwise (k >= 17) the handle times PIPE and
                                 TEAM on its first analysis' first chunk and keeps the faster;
                                 cached per problem shape for the process, so handles of the
@@ -153,9 +154,14 @@ typedef struct letkf_config {
     int32_t precision;         /* LETKF_FP32 or LETKF_MIXED                             */
     int32_t eig_schedule;      /* LETKF_EIG_*; 0 (AUTO) lets the handle choose          */
     int32_t gram_tile;         /* LETKF_GRAM_*; 0 (AUTO) lets the handle choose         */
-    int64_t chunk_bytes;       /* device bytes for the per-point k x k Gram buffer;
-                                  0 = default (1 GiB; larger chunks give the
-                                  thread-per-matrix QL kernel more matrices per launch) */
+    int64_t chunk_bytes;       /* device bytes for the per-point k x k Gram buffer, in whole
+                                  grid rows (1 to 16 of them at least, the CUDA-core
+                                  schedules' tile height); 0 = default (1 GiB; larger chunks
+                                  give the thread-per-matrix QL kernel more matrices per
+                                  launch).  The products of LETKF_GRAM_TENSOR take at most as
+                                  much again (2 GiB with the default); where they, or eight
+                                  rows, do not fit, the schedules that need no products serve
+                                  (LETKF_GRAM_PIPE / TEAM, or LETKF_MIXED's split-FP16 form) */
     void   *stream;            /* cudaStream_t to run on; NULL = a stream the handle
                                   creates and owns                                       */
 } letkf_config;

@@ -36,6 +36,9 @@ constexpr int64_t kDefaultChunkBytes = 1ll << 30;  // 1 GiB: 65,536 points at k 
 // most per pair tile) the CUDA-core schedules stay.
 constexpr int64_t kGemmMaxBytes = 2ll << 30;
 constexpr int kGemmMinPoints = 1024;
+// Its smallest chunk, in rows (of a tile's 16): fewer than these leave more than half of a tile's
+// work unused, and the CUDA-core schedules take chunks of one to twelve rows.
+constexpr int kGemmMinRows = lk::kGemmTile / 2;
 
 // AUTO at k > 64 puts the polynomial transform before the split schedule on chunks of this many
 // points.  It is the faster at every size (k = 80 / 128, kappa some tens: 32 x 32 points 0.16 /
@@ -141,15 +144,27 @@ int make_plan(const letkf_config *c, Plan *p) {
         p->inv2r2 = (float)(1.0 / (2.0 * r * r));
         p->inv_c = (float)(1.0 / (sqrt(10.0 / 3.0) * r));
     }
+    // Gram chunk: rows of the grid that fit chunk_bytes
+    const int64_t budget = c->chunk_bytes > 0 ? c->chunk_bytes : kDefaultChunkBytes;
+    const int64_t row_bytes = (int64_t)c->nx * c->k * c->k * (int64_t)sizeof(float);
+    int rows = (int)std::clamp<int64_t>(budget / row_bytes, 1, c->ny);
     // The Gram matrices as one product over the observation points (gram_gemm.cu): squared
-    // distances exact in FP32, coordinates in 16 bits, and the products of all observation
-    // points within kGemmMaxBytes.
+    // distances exact in FP32, coordinates in 16 bits, the products of all observation points
+    // within kGemmMaxBytes (and within chunk_bytes where it is given), and half a tile of rows
+    // at least (kGemmMinRows) or the whole grid in a chunk.
     p->np = lk::gram_gemm_pairs(c->k);
     const int64_t zbytes = (int64_t)c->n_obs * p->np * 3 * 2;
+    const int64_t zmax = c->chunk_bytes > 0 ? std::min(budget, kGemmMaxBytes) : kGemmMaxBytes;
     p->gemm = c->n_obs > 0 && c->nx < 65536 && c->ny < 65536 &&
-              (c->loc_kind == LETKF_LOC_NONE || p->d2max < (1 << 23)) && zbytes <= kGemmMaxBytes &&
+              (c->loc_kind == LETKF_LOC_NONE || p->d2max < (1 << 23)) && zbytes <= zmax &&
               (p->tensor_gram || c->gram_tile == LETKF_GRAM_AUTO) &&
-              p->npts >= (size_t)kGemmMinPoints;
+              p->npts >= (size_t)kGemmMinPoints && rows >= std::min(kGemmMinRows, c->ny);
+    // whole tiles, or half a tile (the kernel's tiles lie on multiples of their height in the
+    // grid, so a chunk's rows are the same bits for every chunk size)
+    const int unit = !p->gemm ? p->tile_h : rows >= lk::kGemmTile ? lk::kGemmTile : kGemmMinRows;
+    if (rows < c->ny) rows = std::min(c->ny, std::max(unit, rows / unit * unit));
+    p->chunk_rows = rows;
+    p->chunk_pts = (size_t)rows * c->nx;
     if (p->gemm) p->tile_h = std::lcm(p->tile_h, lk::kGemmTile);
     // bins: smallest power-of-two edge (>= 8) whose patch of one Gram tile fits the kernel
     const int maxc = lk::gram_max_cells();
@@ -166,14 +181,6 @@ int make_plan(const letkf_config *c, Plan *p) {
         }
         if (bx * by <= maxc) break;
     }
-    // Gram chunk: whole multiples of the tile height, within chunk_bytes
-    const int64_t budget = c->chunk_bytes > 0 ? c->chunk_bytes : kDefaultChunkBytes;
-    const size_t row_bytes = (size_t)c->nx * c->k * c->k * sizeof(float);
-    int rows = (int)std::max<int64_t>(1, budget / (int64_t)row_bytes);
-    rows = std::max(p->tile_h, rows / p->tile_h * p->tile_h);
-    if (rows >= c->ny) rows = c->ny;
-    p->chunk_rows = rows;
-    p->chunk_pts = (size_t)rows * c->nx;
 
     size_t off = 0;
     auto take = [&](size_t bytes) {

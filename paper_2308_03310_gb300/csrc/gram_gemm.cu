@@ -207,7 +207,7 @@ __device__ __noinline__ void gram_slow(const GemmArgs &a, int tx0, int ty0, int 
     for (int e = threadIdx.x; e < kMT * kPts; e += kThreads) {
         const int m = mt * kMT + e % kMT, n = e / kMT;
         const int off = a.offs[m], px = tx0 + n % kTW, py = ty0 + n / kTW;
-        if (off < 0 || px >= a.nx || py >= a.y_end) continue;
+        if (off < 0 || px >= a.nx || py < a.y_begin || py >= a.y_end) continue;
         float acc = 0.0f;
         for (int r = 0; r < 2 * nyb; ++r) {
             const int yi = r >> 1, by = yi < ly0 ? ry.lo[0] + yi : ry.lo[1] + (yi - ly0);
@@ -247,14 +247,16 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     const ObsNet &net = a.net;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int ntx = (a.nx + kTW - 1) / kTW, nty = (a.y_end - a.y_begin + kTH - 1) / kTH;
+    // tiles lie on multiples of 16 in the grid, so a point's sums do not depend on the chunk
+    const int ty_first = a.y_begin / kTH * kTH;
+    const int ntx = (a.nx + kTW - 1) / kTW, nty = (a.y_end - ty_first + kTH - 1) / kTH;
     const int ntiles = ntx * nty, nmt = a.np / kMT;
     const int nitems = ntiles * nmt;
     // item -> origin of its tile; returns its pair tile
     auto item_at = [&](int it, int &tx0, int &ty0) -> int {
         const int mt = it / ntiles, tile = it - mt * ntiles;
         tx0 = (tile % ntx) * kTW;
-        ty0 = a.y_begin + (tile / ntx) * kTH;
+        ty0 = ty_first + (tile / ntx) * kTH;
         return mt;
     };
 
@@ -593,12 +595,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const size_t stride = off >= kGemmC ? (size_t)a.k : (size_t)a.k * a.k;
                 float *base = off >= kGemmC ? a.cvec + (off - kGemmC) : a.gram + off;
                 const int yb = ty0 + half * (kTH / 2);
-                base += ((size_t)(yb - a.y_begin) * a.nx + tx0) * stride;
+                base += ((ptrdiff_t)(yb - a.y_begin) * a.nx + tx0) * (ptrdiff_t)stride;
                 const bool whole = tx0 + kTW <= a.nx;
 #pragma unroll
                 for (int r = 0; r < kTH / 2; ++r, base += (size_t)a.nx * stride) {
                     float *p = base;
-                    if (yb + r >= a.y_end) continue;
+                    if (yb + r < a.y_begin || yb + r >= a.y_end) continue;
 #pragma unroll
                     for (int i = 0; i < kTW; ++i, p += stride)
                         if (whole || tx0 + i < a.nx) *p = acc[kTW * r + i];
@@ -752,7 +754,7 @@ cudaError_t launch_gram_gemm(const GemmArgs &a, const TmaMap &map, int *status, 
                              cudaStream_t s) {
     if (a.y_end <= a.y_begin) return cudaSuccess;
     const long long tiles = (long long)((a.nx + kTW - 1) / kTW) *
-                            ((a.y_end - a.y_begin + kTH - 1) / kTH);
+                            ((a.y_end - a.y_begin / kTH * kTH + kTH - 1) / kTH);
     const long long items = tiles * (a.np / kMT);
     int lo = 0, hi = 0;
     cudaError_t e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
