@@ -71,7 +71,8 @@ struct Plan {
     float inv_c = 0.0f;  // Gaspari-Cohn: 1 / (sqrt(10/3) r)
     // byte offsets inside the workspace
     size_t off_state[2], off_force, off_xg, off_obs_xy, off_cell_start, off_cell_obs, off_rinv,
-        off_yf, off_yb, off_ybar, off_yo, off_orec, off_z, off_oxy, off_pairs, off_offs, off_gram, off_cvec, off_nloc, off_nloc_all,
+        off_yf, off_yb, off_ybar, off_yo, off_orec, off_z, off_zbad, off_oxy, off_pairs,
+        off_offs, off_gram, off_cvec, off_nloc, off_nloc_all,
         off_eigval, off_de, off_taus, off_rot, off_nrot, off_list, off_pre_list, off_status,
         total;
 };
@@ -204,6 +205,7 @@ int make_plan(const letkf_config *c, Plan *p) {
     p->off_yo = take((size_t)p->LV * sizeof(float));
     p->off_orec = take(p->tensor_gram ? (size_t)p->LV * sizeof(float4) : 0);
     p->off_z = take(p->gemm ? (size_t)zbytes : 0);
+    p->off_zbad = take(p->gemm ? (size_t)c->n_obs * sizeof(int) : 0);
     p->off_oxy = take(p->gemm ? (size_t)c->n_obs * sizeof(float2) : 0);
     p->off_pairs = take(p->gemm ? (size_t)p->np * sizeof(int) : 0);
     p->off_offs = take(p->gemm ? (size_t)p->np * sizeof(int) : 0);
@@ -261,7 +263,7 @@ struct letkf_handle {
     bool gemm = false;            // the one-product Gram form is in use
     __nv_bfloat16 *z = nullptr;   // its products, observation points, pair tables, tensor map
     float2 *oxy = nullptr;
-    int *pairs = nullptr, *offs = nullptr;
+    int *zbad = nullptr, *pairs = nullptr, *offs = nullptr;
     lk::TmaMap zmap;
     int2 *obs_xy = nullptr;
     int *cell_start = nullptr, *cell_obs = nullptr, *nloc = nullptr, *nloc_all = nullptr,
@@ -454,14 +456,22 @@ int enqueue_gram_chunk(letkf_handle *h, int chunk, int y0, int y1) {
         m.k = h->cfg.k;
         m.y_begin = y0;
         m.y_end = y1;
+        m.kp = g.kp;
+        m.yb = g.yb;
+        m.ybar = g.ybar;
+        m.yo = g.yo;
+        m.rinv = g.rinv;
+        std::copy(g.yref, g.yref + 3, m.yref);
         m.oxy = h->oxy;
+        m.pairs = h->pairs;
         m.offs = h->offs;
         m.z = h->z;
         m.np = h->plan.np;
         m.gram = h->gram;
         m.cvec = h->cvec;
+        m.zbad = h->zbad;
         m.flag = h->status + kGemmFlag;
-        if (chunk == 0) CK(lk::launch_gram_z(m, g, h->pairs, h->stream));
+        if (chunk == 0) CK(lk::launch_gram_z(m, h->stream));
         CK(lk::launch_gram_gemm(m, h->zmap, h->status, h->tc_ctas, h->stream));
         return LETKF_OK;
     }
@@ -1089,6 +1099,7 @@ int letkf_init(const letkf_config *cfg, void *workspace, size_t workspace_bytes,
     h->orec = plan.tensor_gram ? (float4 *)(w + plan.off_orec) : nullptr;
     if (plan.gemm) {
         h->z = (__nv_bfloat16 *)(w + plan.off_z);
+        h->zbad = (int *)(w + plan.off_zbad);
         h->oxy = (float2 *)(w + plan.off_oxy);
         h->pairs = (int *)(w + plan.off_pairs);
         h->offs = (int *)(w + plan.off_offs);

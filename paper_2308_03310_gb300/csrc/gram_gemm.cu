@@ -41,9 +41,11 @@
 // Every wait is bounded in time: on expiry the status word gets ST_TIMEOUT, all roles leave, the
 // copies and MMAs in flight are awaited (bounded) and the tensor memory is freed.
 //
-// A non-finite dy or innovation would reach every point of a tile through 0 x inf; gram_z_kernel
-// then raises a flag and the launch takes gram_slow() instead, which adds only the observations
-// within each point's cutoff.
+// A non-finite product would reach every point of a tile through 0 x inf: gram_z_kernel puts zeros
+// in its place and marks the row, and gram_fix() adds the marked rows' non-finite products to the
+// points within their cutoff, after the sums are stored and only in tiles whose patch holds such a
+// row.  Gram phase at 256^2, k = 64, r = 12: finite 0.97 ms, one NaN observation 1.16, a whole member
+// NaN 2.5 (every point's own observations summed per entry in such a case: 372 ms).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -196,39 +198,120 @@ __device__ __forceinline__ BinRanges patch_rows(const ObsNet &net, int ny, int t
     return ry;
 }
 
-// The work item's sums in plain FP32, only over each point's own local observations: taken
-// where some z is not finite.
+// One entry of z in two FP32 words (compensated): the sum over the observed variables of
+// dy_i dy_j / sigma^2, from f(v) = (dy_vi, dy_vj, 1 / sigma_v^2).
+template <class F>
+__device__ __forceinline__ void z_entry(int V, F f, float &hi, float &lo) {
+    float acc = 0.0f, err = 0.0f;
+    for (int v = 0; v < V; ++v) {
+        const float3 d = f(v);
+        const float t = d.x * d.y;
+        const float e = fmaf(d.x, d.y, -t);
+        const float t2 = t * d.z;
+        const float e2 = fmaf(e, d.z, fmaf(t, d.z, -t2));
+        const float s = acc + t2, b = s - acc;
+        err += ((acc - (s - b)) + (t2 - b)) + e2;
+        acc = s;
+    }
+    hi = acc + err;
+    lo = err - (hi - acc);
+    if (!isfinite(hi)) {   // the plain sum keeps an overflowed error term out
+        hi = acc;
+        lo = 0.0f;
+    }
+}
+
+// Whether the products take v as it is (its first BF16 part is finite).
+__device__ __forceinline__ bool z_finite(float v) {
+    return isfinite(__bfloat162float(__float2bfloat16_rn(v)));
+}
+
+// dy_i of observation o's variable v (i < k), or its innovation (i = k).
+__device__ __forceinline__ float z_factor(const GemmArgs &a, int o, int v, int i) {
+    const int s = o * a.net.V + v;
+    return i < a.k ? a.yb[(size_t)s * a.kp + i] : (a.yo[s] - a.yref[v]) - a.ybar[s];
+}
+
+// Adds the products that gram_z_kernel left out (not finite) to the entries of a warp's 32 pairs and
+// 8 rows of a tile, which its lanes have stored: the rows of the patch, 32 at a time, from the
+// middle of the patch and of each run (near every point), until every entry is a NaN.  A NaN is
+// stored without a look at the sum, so that nothing waits for a load.
 template <int KIND>
-__device__ __noinline__ void gram_slow(const GemmArgs &a, int tx0, int ty0, int mt) {
-    const ObsNet &net = a.net;
-    const BinRanges ry = patch_rows(net, a.ny, ty0);
+__device__ __noinline__ void gram_fix(const GemmArgs &a, int tx0, int ty0, int mt, int warp,
+                                      int lane) {
+    const ObsNet net = a.net;   // (copies: a is in memory here, and the stores might alias it)
+    const int nx = a.nx, ny = a.ny, y_begin = a.y_begin, y_end = a.y_end, k = a.k;
+    const int *const zbad = a.zbad;
+    const float2 *const oxy = a.oxy;
+    const int m = mt * kMT + 32 * (warp & 3) + lane, off = a.offs[m], pr = a.pairs[m];
+    const int yb = ty0 + ((warp - kWarpSum) >> 2) * (kTH / 2);
+    const size_t stride = off >= kGemmC ? (size_t)k : (size_t)k * k;
+    float *const base = off >= kGemmC ? a.cvec + (off - kGemmC) : a.gram + off;
+    uint32_t todo[kTH / 4];   // a bit per point (two rows per word), cleared once it is a NaN
+#pragma unroll
+    for (int wd = 0; wd < kTH / 4; ++wd) {
+        const int y = yb + 2 * wd;
+        const uint32_t row = off < 0 || tx0 >= nx ? 0u : 0xffffu >> max(0, tx0 + kTW - nx);
+        todo[wd] = (y >= y_begin && y < y_end ? row : 0u) |
+                   (y + 1 >= y_begin && y + 1 < y_end ? row << kTW : 0u);
+    }
+    const BinRanges ry = patch_rows(net, ny, ty0);
     const int ly0 = ry.hi[0] - ry.lo[0] + 1;
     const int nyb = ly0 + (ry.n > 1 ? ry.hi[1] - ry.lo[1] + 1 : 0);
-    for (int e = threadIdx.x; e < kMT * kPts; e += kThreads) {
-        const int m = mt * kMT + e % kMT, n = e / kMT;
-        const int off = a.offs[m], px = tx0 + n % kTW, py = ty0 + n / kTW;
-        if (off < 0 || px >= a.nx || py < a.y_begin || py >= a.y_end) continue;
-        float acc = 0.0f;
-        for (int r = 0; r < 2 * nyb; ++r) {
+    for (int rb = 0; rb < 2 * nyb; rb += 32) {     // 32 runs at a time, one per lane
+        int r = rb + lane + nyb, run0 = 0, runn = 0;
+        r -= r >= 2 * nyb ? 2 * nyb : 0;
+        if (rb + lane < 2 * nyb) {
             const int yi = r >> 1, by = yi < ly0 ? ry.lo[0] + yi : ry.lo[1] + (yi - ly0);
-            int j0 = 0;
-            const int cnt = patch_run(net, a.nx, a.ny, tx0, ty0, by, r & 1, &j0);
-            for (int j = j0; j < j0 + cnt; ++j) {
-                const float2 o = a.oxy[j];
-                const int dx = min_image((int)o.x - px, a.nx), dy = min_image((int)o.y - py, a.ny);
-                const int d2 = dx * dx + dy * dy;
-                if (KIND != 0 && d2 > net.d2max) continue;
-                float z = 0.0f;
-                for (int s = 2; s >= 0; --s)
-                    z += __bfloat162float(a.z[((size_t)s * net.L + j) * a.np + m]);
-                // a part beyond BF16's range leaves inf - inf in the lower parts: take the first
-                const float h = __bfloat162float(a.z[(size_t)j * a.np + m]);
-                acc = fmaf(weight_d2<KIND>(net, (float)d2), isfinite(h) ? z : h, acc);
+            runn = patch_run(net, nx, ny, tx0, ty0, by, r & 1, &run0);
+        }
+        for (unsigned runs = __ballot_sync(0xffffffffu, runn > 0); runs; runs &= runs - 1) {
+            const int j0 = __shfl_sync(0xffffffffu, run0, __ffs(runs) - 1);
+            const int cnt = __shfl_sync(0xffffffffu, runn, __ffs(runs) - 1);
+            for (int c = 0; c < cnt; c += 32) {
+                int jl = j0 + cnt / 2 + c + lane;
+                jl -= jl >= j0 + cnt ? cnt : 0;
+                unsigned marked = __ballot_sync(0xffffffffu, c + lane < cnt && zbad[jl]);
+                for (; marked; marked &= marked - 1) {
+                    const int j = __shfl_sync(0xffffffffu, jl, __ffs(marked) - 1);
+                    const int o = net.cell_obs[j];
+                    float v = 0.0f, lo = 0.0f;
+                    if (off >= 0)
+                        z_entry(net.V, [&](int w) {
+                            return make_float3(z_factor(a, o, w, pr & 0xffff),
+                                               z_factor(a, o, w, pr >> 16), a.rinv[o * net.V + w]);
+                        }, v, lo);
+                    const bool add = !z_finite(v), nan = isnan(v);
+                    if (!__any_sync(0xffffffffu, add)) continue;
+                    const float2 at = oxy[j];
+#pragma unroll
+                    for (int wd = 0; wd < kTH / 4; ++wd)
+#pragma unroll 1
+                        for (int h = 0; h < 2; ++h) {
+                            const int y = yb + 2 * wd + h, dy = min_image((int)at.y - y, ny);
+                            if (KIND != 0 && dy * dy > net.d2max) continue;
+                            float *const row = base + ((ptrdiff_t)(y - y_begin) * nx + tx0) *
+                                                          (ptrdiff_t)stride;
+#pragma unroll 1
+                            for (int i = 0; i < kTW; ++i) {
+                                const int dx = min_image((int)at.x - (tx0 + i), nx);
+                                const int d2 = dx * dx + dy * dy;
+                                const uint32_t bit = 1u << (h * kTW + i);
+                                if ((KIND != 0 && d2 > net.d2max) || !add || !(todo[wd] & bit))
+                                    continue;
+                                float t = v;
+                                if (!nan) t = fmaf(weight_d2<KIND>(net, (float)d2), v, row[i * stride]);
+                                row[i * stride] = t;
+                                if (isnan(t)) todo[wd] &= ~bit;
+                            }
+                        }
+                    uint32_t left = 0;
+#pragma unroll
+                    for (int wd = 0; wd < kTH / 4; ++wd) left |= todo[wd];
+                    if (!__any_sync(0xffffffffu, left != 0)) return;
+                }
             }
         }
-        const size_t lp = (size_t)(py - a.y_begin) * a.nx + px;
-        if (off >= kGemmC) a.cvec[lp * a.k + (off - kGemmC)] = acc;
-        else a.gram[lp * a.k * a.k + off] = acc;
     }
 }
 
@@ -259,15 +342,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         ty0 = ty_first + (tile / ntx) * kTH;
         return mt;
     };
-
-    if (*a.flag) {   // written before this launch; the same for every thread
-        for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-            int tx0, ty0;
-            const int mt = item_at(it, tx0, ty0);
-            gram_slow<KIND>(a, tx0, ty0, mt);
-        }
-        return;
-    }
 
     if (tid == 0) {
         for (int i = 0; i < kNM; ++i) {
@@ -608,6 +682,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
         if (!ok) fail();
+        else if (*a.flag)   // written before this launch; the lanes' own stores are the operands
+            for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
+                int tx0, ty0;
+                const int mt = item_at(it, tx0, ty0);
+                gram_fix<KIND>(a, tx0, ty0, mt, warp, lane);
+            }
     }
 
     // ---- stop: every role has left its loop; free the tensor memory
@@ -621,64 +701,49 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // z of every observation point in bin order, three BF16 parts: block per observation point, two
 // neighbouring pairs per thread and round.  pairs[m] = i | j << 16 (j = k: the innovation), -1:
-// padding.  The sum over the observed variables is carried in two FP32 words.
-__global__ void __launch_bounds__(256) gram_z_kernel(ObsNet net, int k, int kp,
-                                                     const float *yb, const float *ybar,
-                                                     const float *yo, const float *rinv,
-                                                     float r0, float r1, float r2,
-                                                     const int *pairs, int np,
-                                                     __nv_bfloat16 *z, int *flag) {
+// padding.  An entry that is not finite becomes zero; its row is marked in zbad, and the flag raised.
+__global__ void __launch_bounds__(256) gram_z_kernel(const __grid_constant__ GemmArgs a) {
     __shared__ float dy[3][132];
     __shared__ float ri[3];
-    const int j = blockIdx.x, o = net.cell_obs[j], V = net.V;
+    const int j = blockIdx.x, o = a.net.cell_obs[j], V = a.net.V, k = a.k, np = a.np;
     for (int e = threadIdx.x; e < V * (k + 1); e += blockDim.x) {
-        const int v = e / (k + 1), i = e - v * (k + 1), s = o * V + v;
-        const float ref = v == 0 ? r0 : (v == 1 ? r1 : r2);
-        dy[v][i] = i < k ? yb[(size_t)s * kp + i] : (yo[s] - ref) - ybar[s];
+        const int v = e / (k + 1), i = e - v * (k + 1);
+        dy[v][i] = z_factor(a, o, v, i);
     }
-    if (threadIdx.x < V) ri[threadIdx.x] = rinv[o * V + threadIdx.x];
+    if (threadIdx.x < V) ri[threadIdx.x] = a.rinv[o * V + threadIdx.x];
     __syncthreads();
     bool bad = false;
     for (int m = 2 * threadIdx.x; m < np; m += 2 * blockDim.x) {
-        const int2 pr = *reinterpret_cast<const int2 *>(pairs + m);
+        const int2 pr = *reinterpret_cast<const int2 *>(a.pairs + m);
         float hi[2], lo[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int p = h ? pr.y : pr.x;
-            float acc = 0.0f, err = 0.0f;
-            if (p >= 0) {
-                const int i = p & 0xffff, jj = p >> 16;
-                for (int v = 0; v < V; ++v) {
-                    const float t = dy[v][i] * dy[v][jj];
-                    const float e = fmaf(dy[v][i], dy[v][jj], -t);
-                    const float t2 = t * ri[v];
-                    const float e2 = fmaf(e, ri[v], fmaf(t, ri[v], -t2));
-                    const float s = acc + t2, b = s - acc;
-                    err += ((acc - (s - b)) + (t2 - b)) + e2;
-                    acc = s;
-                }
-            }
-            hi[h] = acc + err;
-            lo[h] = err - (hi[h] - acc);
-            bad |= !isfinite(hi[h]);
-            if (!isfinite(hi[h])) {   // the plain sum keeps an overflowed error term out
-                hi[h] = acc;
-                lo[h] = 0.0f;
+            hi[h] = lo[h] = 0.0f;
+            if (p >= 0)
+                z_entry(V, [&](int v) { return make_float3(dy[v][p & 0xffff], dy[v][p >> 16], ri[v]); },
+                        hi[h], lo[h]);
+            if (!z_finite(hi[h])) {
+                bad = true;
+                hi[h] = lo[h] = 0.0f;
             }
         }
         const __nv_bfloat162 hb = __floats2bfloat162_rn(hi[0], hi[1]);
         const float2 hf = bf2f(hb);
-        bad |= !isfinite(hf.x) || !isfinite(hf.y);
         const float a0 = (hi[0] - hf.x) + lo[0], a1 = (hi[1] - hf.y) + lo[1];
         const __nv_bfloat162 mb = __floats2bfloat162_rn(a0, a1);
         const float2 mf = bf2f(mb);
         const __nv_bfloat162 lb = __floats2bfloat162_rn(a0 - mf.x, a1 - mf.y);
-        const size_t part = (size_t)net.L * np, at = (size_t)j * np + m;
-        *reinterpret_cast<__nv_bfloat162 *>(z + at) = hb;
-        *reinterpret_cast<__nv_bfloat162 *>(z + part + at) = mb;
-        *reinterpret_cast<__nv_bfloat162 *>(z + 2 * part + at) = lb;
+        const size_t part = (size_t)a.net.L * np, at = (size_t)j * np + m;
+        *reinterpret_cast<__nv_bfloat162 *>(a.z + at) = hb;
+        *reinterpret_cast<__nv_bfloat162 *>(a.z + part + at) = mb;
+        *reinterpret_cast<__nv_bfloat162 *>(a.z + 2 * part + at) = lb;
     }
-    if (bad) atomicOr(flag, 1);
+    const int any = __syncthreads_or(bad);
+    if (threadIdx.x == 0) {
+        a.zbad[j] = any;
+        if (any) atomicOr(a.flag, 1);
+    }
 }
 
 using EncodeTiled = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
@@ -743,10 +808,9 @@ cudaError_t gram_gemm_prepare(const void *z, int L, int np, TmaMap *map, int *ok
     return cudaSuccess;
 }
 
-cudaError_t launch_gram_z(const GemmArgs &a, const GramArgs &g, const int *pairs, cudaStream_t s) {
+cudaError_t launch_gram_z(const GemmArgs &a, cudaStream_t s) {
     if (a.net.L <= 0) return cudaSuccess;
-    gram_z_kernel<<<a.net.L, 256, 0, s>>>(a.net, a.k, g.kp, g.yb, g.ybar, g.yo, g.rinv, g.yref[0],
-                                          g.yref[1], g.yref[2], pairs, a.np, a.z, a.flag);
+    gram_z_kernel<<<a.net.L, 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -105,18 +105,23 @@ struct GemmArgs {
     ObsNet net;
     int nx, ny, k;
     int y_begin, y_end;     // grid rows of this chunk
+    int kp;                 // the inputs, as in GramArgs
+    const float *yb, *ybar, *yo, *rinv;
+    float yref[3];
     const float2 *oxy;      // [L] observation points in bin order
+    const int *pairs;       // [np] a pair's members i | j << 16 (j = k: the innovation), -1: padding
     const int *offs;        // [np] a pair's offset in the k x k slot, or in c, or -1 (padding)
     __nv_bfloat16 *z;       // [3][L][np] the pairs' products, three parts, rows in bin order
     int np;                 // pairs, padded (gram_gemm_pairs)
     float *gram, *cvec;     // as in GramArgs
-    int *flag;              // raised by launch_gram_z where some product is not finite
+    int *zbad;              // [L] 1: a row with products that are not finite (zero in z)
+    int *flag;              // raised by launch_gram_z where there is such a row
 };
 int gram_gemm_pairs(int k);
 void gram_gemm_tables(int k, int *pairs, int *offs);   // [gram_gemm_pairs(k)] each
 // the tensor map of z; *ok = 0 where the driver offers no encoder
 cudaError_t gram_gemm_prepare(const void *z, int L, int np, TmaMap *map, int *ok);
-cudaError_t launch_gram_z(const GemmArgs &a, const GramArgs &g, const int *pairs, cudaStream_t s);
+cudaError_t launch_gram_z(const GemmArgs &a, cudaStream_t s);
 cudaError_t launch_gram_gemm(const GemmArgs &a, const TmaMap &map, int *status, int max_ctas,
                              cudaStream_t s);
 
