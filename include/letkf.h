@@ -112,8 +112,10 @@ extern "C" {
 #define LETKF_GRAM_AUTO   0  /* LETKF_GRAM_TENSOR from 1,024 grid points on, where the network's
                                 products (n_obs x k (k + 3) / 2 entries of 6 bytes) fit in 2
                                 GiB and in letkf_config.chunk_bytes, eight grid rows (or the
-                                grid) in a chunk, and coordinates and cutoff are below 65536
-                                and 2896 cells.  Otherwise (k >= 17) the handle times PIPE and
+                                grid) in a chunk, coordinates and cutoff are below 65536 and
+                                2896 cells, and (k >= 17) it is estimated to be the faster form:
+                                not on grids one or two points wide, nor with cutoffs of a few
+                                cells on dense networks.  Otherwise (k >= 17) the handle times PIPE and
                                 TEAM on its first analysis' first chunk and keeps the faster;
                                 cached per problem shape for the process, so handles of the
                                 same shape run the same arithmetic                          */

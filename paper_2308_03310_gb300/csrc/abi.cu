@@ -36,8 +36,10 @@ constexpr int64_t kDefaultChunkBytes = 1ll << 30;  // 1 GiB: 65,536 points at k 
 // most per pair tile) the CUDA-core schedules stay.
 constexpr int64_t kGemmMaxBytes = 2ll << 30;
 constexpr int kGemmMinPoints = 1024;
-// Its smallest chunk, in rows (of a tile's 16): fewer than these leave more than half of a tile's
-// work unused, and the CUDA-core schedules take chunks of one to twelve rows.
+// Its smallest chunk, in rows (of a tile's 16).  Chunks of eight rows of 256 x 128 points, every
+// fourth observed, r = 3 / 12: k = 32 0.30 / 0.64 ms against 0.41 / 2.30 (LETKF_MIXED 0.33 / 1.33),
+// k = 64 0.42 / 1.13 against 0.57 / 3.16 (0.64 / 2.14), k = 100 0.83 / 2.5 against 1.9 / 18.7 (1.2 /
+// 7.2); fewer rows leave more than half of a tile's work unused.
 constexpr int kGemmMinRows = lk::kGemmTile / 2;
 
 // AUTO at k > 64 puts the polynomial transform before the split schedule on chunks of this many
@@ -109,6 +111,55 @@ int validate(const letkf_config *c) {
     return LETKF_OK;
 }
 
+// Whether the one-product Gram form is the faster one, from the sizes alone (the network by its mean
+// density), k >= 17: on grids one or two points wide most of a tile's 256 points are unused, and with a
+// short cutoff on a dense network most of its observations are local to few of them.
+// Estimates in ns per grid point, fitted to the Gram phase of 390 shapes (k = 24, 40, 64, 128; 160 x 160
+// and 96 x 96 points observed at every, every second and fourth one, r = 0.5 to 6, one to three
+// variables; 8192 x 1 to 1024 x 11 and their transposes): the slower form is taken in 16 of them, by
+// 0.08 ms at most.  Where the other forms win: 8192 x 1, k = 64 / 128 0.11 / 0.33 ms against 0.21 /
+// 0.72, every point of 160 x 160 observed with r = 1, k = 64 0.59 (LETKF_MIXED 0.44) against 0.71;
+// where they lose: 2048 x 3, k = 64 0.084 against 0.079, r = 2 1.44 (0.81) against 0.72, r = 6 9.4
+// (5.4) against 2.1.  k <= 16: the one-product form is the faster on all but grids one or two points
+// wide, by more in the tests' range than it loses there (5 us of 14 to 24).
+bool gemm_pays(const letkf_config *c, const Plan &p) {
+    if (c->loc_kind == LETKF_LOC_NONE || p.kp < 32 || p.d2max < 0) return true;
+    const int T = lk::kGemmTile, cs = 8;
+    const double density = (double)c->n_obs / (double)p.npts;
+    auto reach = [&](double rem) { return (int)sqrt(rem); };
+    // slots of a tile: per row of bins the observations in the bins its cutoff reaches, in groups of 8
+    double groups = 0.0;
+    int left = c->ny;
+    auto bin_row = [&](int w) {
+        const int h = std::min(cs, left);
+        if (h <= 0) return;
+        const double width = std::min<double>(c->nx, T + 2.0 * cs * ((w + cs - 1) / cs));
+        groups += density * h * width / 8.0 + 0.5;
+        left -= h;
+    };
+    for (int i = 0; i < T / cs; ++i) bin_row(p.cr);
+    for (int g = 1; g <= p.cr && left > 0; g += cs)
+        for (int side = 0; side < 2; ++side) bin_row(reach((double)p.d2max - (double)g * g));
+    const double steps = std::max(1.0, groups / 4.0);
+    const double tiles = (double)((c->nx + T - 1) / T) * ((c->ny + T - 1) / T);
+    const double pairs = p.np / 128.0;
+    const double gemm = 32.0 * (steps + 1.6) * tiles / (double)p.npts * (0.26 * pairs + 0.3) +
+                        0.35 * density * pairs;
+    // the other forms: a term per point and one per local observed scalar
+    double area = 0.0;
+    const int rows = std::min(2 * p.cr + 1, c->ny);
+    for (int i = 0; i < rows; ++i) {
+        const double y = i - rows / 2;
+        area += std::min<double>(c->nx, 2.0 * reach(std::max(0.0, p.d2max - y * y)) + 1.0);
+    }
+    const int kind = p.kp == 32 ? 0 : p.kp == 64 ? 1 : 2;
+    constexpr double point[2][3] = {{4.6, 9.5, 33.0}, {6.0, 9.8, 17.0}};
+    constexpr double scalar[2][3] = {{0.042, 0.125, 0.75}, {0.047, 0.055, 0.26}};
+    const double other =
+        point[p.tensor_gram][kind] + scalar[p.tensor_gram][kind] * p.V * area * density;
+    return gemm <= other;
+}
+
 int make_plan(const letkf_config *c, Plan *p) {
     const int rc = validate(c);
     if (rc != LETKF_OK) return rc;
@@ -159,7 +210,8 @@ int make_plan(const letkf_config *c, Plan *p) {
     p->gemm = c->n_obs > 0 && c->nx < 65536 && c->ny < 65536 &&
               (c->loc_kind == LETKF_LOC_NONE || p->d2max < (1 << 23)) && zbytes <= zmax &&
               (p->tensor_gram || c->gram_tile == LETKF_GRAM_AUTO) &&
-              p->npts >= (size_t)kGemmMinPoints && rows >= std::min(kGemmMinRows, c->ny);
+              p->npts >= (size_t)kGemmMinPoints && rows >= std::min(kGemmMinRows, c->ny) &&
+              gemm_pays(c, *p);
     // whole tiles, or half a tile (the kernel's tiles lie on multiples of their height in the
     // grid, so a chunk's rows are the same bits for every chunk size)
     const int unit = !p->gemm ? p->tile_h : rows >= lk::kGemmTile ? lk::kGemmTile : kGemmMinRows;
