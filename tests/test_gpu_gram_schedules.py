@@ -1,5 +1,8 @@
-"""Which Gram form AUTO takes by the sizes alone; the counts, A (1e-5 relative L2 per point) and the
-analysis (1e-5) against the FP64 oracle."""
+"""Which Gram form AUTO takes by the sizes alone, and the forms without products on problems of several
+tiles per block: LETKF_MIXED's split-FP16 form on 1,023 grid points (a tile is one to eight of
+them), the CUDA-core schedules by name, and both where the one-product form's buffer would be
+beyond 2 GiB.  The counts, A (1e-5 relative L2 per point) and the analysis (1e-5) against the FP64
+oracle."""
 import numpy as np
 import pytest
 
@@ -68,3 +71,21 @@ TENSOR = (L.LETKF_GRAM_TENSOR,)
 def test_auto_picks_the_form_by_its_sizes(nx, ny, k, stride, radius, tiles, precision):
     _check(nx, ny, k, stride, radius, TENSOR if precision == L.LETKF_MIXED else tiles,
            precision=precision)
+
+
+@pytest.mark.parametrize("k", [20, 40, 64, 65, 128])
+def test_mixed_below_the_one_product_forms_grid_size(k):
+    _check(31, 33, k, 3, 3.0, (L.LETKF_GRAM_TENSOR,), precision=L.LETKF_MIXED)
+
+
+@pytest.mark.parametrize("tile", [L.LETKF_GRAM_PIPE, L.LETKF_GRAM_TEAM])
+@pytest.mark.parametrize("nx,ny,k", [(161, 130, 20), (112, 96, 64), (72, 64, 128)])
+def test_cuda_core_schedules_by_name(nx, ny, k, tile):
+    _check(nx, ny, k, 4, 4.0, (tile,), gram_tile=tile)
+
+
+@pytest.mark.parametrize("precision", [L.LETKF_FP32, L.LETKF_MIXED])
+def test_networks_whose_products_exceed_the_buffer(precision):
+    k, nx, ny = 128, 256, 164               # every point observed: 2.16e9 bytes
+    _check(nx, ny, k, 1, 2.0, TENSOR if precision == L.LETKF_MIXED else CORES,
+           precision=precision, eig_schedule=L.LETKF_EIG_FUSED)
