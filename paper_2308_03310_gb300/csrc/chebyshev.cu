@@ -868,11 +868,13 @@ __global__ void __launch_bounds__(32 * ChebBlock::NW, 2)
 #pragma unroll
         for (int t = 0; t < NE; ++t) {
             const int s = NE * w + t, row = s / CS, col = 32 * (s % CS) + lane;
-            float v = mean[t];
+            float v = 0.0f;
 #pragma unroll
             for (int q = 0; q < CS; ++q) v += dots[row * CS + q];
             if (row < NV && col < k) {
-                v = fmaf(sc, Bc[t], v);
+                // the mean last: a rounded sum of mean and increment would be the same error in
+                // every member, and so in the analysis mean
+                v = mean[t] + fmaf(sc, Bc[t], v);
                 bad |= !isfinite(v);
                 X[row * k + col] = v;
             }
