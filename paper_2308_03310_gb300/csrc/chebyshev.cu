@@ -872,9 +872,11 @@ __global__ void __launch_bounds__(32 * ChebBlock::NW, 2)
 #pragma unroll
             for (int q = 0; q < CS; ++q) v += dots[row * CS + q];
             if (row < NV && col < k) {
-                // the mean last: a rounded sum of mean and increment would be the same error in
-                // every member, and so in the analysis mean
-                v = mean[t] + fmaf(sc, Bc[t], v);
+                // mean and increment as two words: their rounded sum alone would be the same error
+                // in every member, and so in the analysis mean
+                const float s0 = mean[t] + v, b0 = s0 - mean[t];
+                const float lo = (mean[t] - (s0 - b0)) + (v - b0);
+                v = s0 + fmaf(sc, Bc[t], lo);
                 bad |= !isfinite(v);
                 X[row * k + col] = v;
             }
