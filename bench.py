@@ -240,19 +240,28 @@ def eigen_flops_per_point(k, schedule):
 
 
 def cheb_flops(k, counts):
-    """Flops of the CHEBYSHEV schedule for the given counts (points, products, handed on):
+    """Flops of the polynomial transform for the given counts (points, products, handed on):
     each product R A of the ten rows with the k x k Gram matrix is 20 k^2 flops, the final
-    increment and combination 4 k per row; the points passed on cost the RATIONAL count."""
+    increment and combination 4 k per row; the points passed on cost the RATIONAL count (k > 64:
+    the SPLIT count)."""
     return (20.0 * k * k * counts["cheb_products"] + 36.0 * k * counts["cheb_points"]
-            + eigen_flops_per_point(k, 4) * counts["cheb_handed_on"])
+            + eigen_flops_per_point(k, 4 if k <= 64 else 2) * counts["cheb_handed_on"])
+
+
+def polynomial_transform(k, schedule, counts):
+    """Whether the eigen phase ran the polynomial transform: the CHEBYSHEV schedule, and for
+    k > 64 AUTO's SPLIT with the transform before it (its counters have advanced)."""
+    return schedule == 5 or (schedule == 2 and k > 64 and bool(counts)
+                             and counts["cheb_points"] + counts["cheb_handed_on"] > 0)
 
 
 def kernel_work(w, k, npts, mean_local_obs, V, nobs_pts, chunks, steps, schedule=1,
                 cheb_counts=None, steps_per_launch=2):
-    """Algorithmic work of one cycle per kernel: (unit, amount, launches).  For the CHEBYSHEV
-    schedule the eigen phase's work follows the device counters of the cycle (cheb_counts);
-    without them it falls back to the RATIONAL count."""
-    eig = (cheb_flops(k, cheb_counts) if schedule == 5 and cheb_counts
+    """Algorithmic work of one cycle per kernel: (unit, amount, launches).  Where the polynomial
+    transform ran the eigen phase's work follows the device counters of the cycle
+    (cheb_counts); without them the CHEBYSHEV schedule falls back to the RATIONAL count."""
+    eig = (cheb_flops(k, cheb_counts)
+           if cheb_counts and polynomial_transform(k, schedule, cheb_counts)
            else eigen_flops_per_point(k, schedule) * npts)
     return {
         # one read and one write of the state (+ the force) per launch of steps_per_launch steps
@@ -1569,7 +1578,7 @@ def measure(w, members, setup, yos, device, precision, steps, warm, world, eig_s
                       "zero_fraction": st.n_zero_obs / st.n_points},
         **({"chebyshev_per_cycle": {**cheb, "mean_degree": (cheb["cheb_products"]
                                                             / max(cheb["cheb_points"], 1))}}
-           if st_end.eig_schedule == L.LETKF_EIG_CHEBYSHEV else {}),
+           if polynomial_transform(w.k, st_end.eig_schedule, cheb) else {}),
     }
 
 
