@@ -57,20 +57,23 @@ extern "C" {
                                   (the default cutoff of LETKF_LOC_GAUSS); the cutoff is
                                   capped at 2c, so every local observation has G > 0   */
 
-#define LETKF_FP32  0          /* plain FP32 CUDA-core analysis                                */
-#define LETKF_MIXED 1          /* split-precision: for 17 <= k <= 128 the localized Gram runs on
-                                  the tensor cores on every grid (from 1,024 grid points on as
-                                  LETKF_GRAM_TENSOR below; on smaller ones with FP16 hi+lo
-                                  operands and FP32 accumulation; for k <= 32 two grid points
-                                  share one operand tile); for k <= 16 as in LETKF_FP32     */
+#define LETKF_FP32  0          /* FP32 accuracy throughout: the localized Gram on CUDA cores or,
+                                  where LETKF_GRAM_AUTO takes LETKF_GRAM_TENSOR, on the tensor
+                                  cores with 24 significant bits per operand               */
+#define LETKF_MIXED 1          /* split precision where it pays: the Gram as in LETKF_FP32 where
+                                  that takes LETKF_GRAM_TENSOR (the same kernel and bits) and for
+                                  k <= 16; elsewhere, for 17 <= k <= 128, on the tensor cores
+                                  with FP16 hi+lo operands and FP32 accumulation (for k <= 32
+                                  two grid points share one operand tile)                  */
 
 /* Eigensolve schedules (same results up to rounding; see letkf_config.eig_schedule). */
 #define LETKF_EIG_AUTO        0  /* the handle picks one: at its first analysis the schedules
                                     (FUSED, SPLIT and, for k <= 64, CHEBYSHEV, which passes its
                                     ill-conditioned points to RATIONAL; for k > 64, on chunks of
                                     4,096 points and more, SPLIT with CHEBYSHEV's transform
-                                    before it for the points with kappa up to 400, named SPLIT in
-                                    letkf_stats) are timed on
+                                    before it for the points with kappa up to 80 (k = 65), 180
+                                    (k = 100), 400 (k = 128), named SPLIT in letkf_stats, although
+                                    SPLIT by name has no such transform) are timed on
                                     that analysis' first chunk of Gram matrices
                                     (applied to a scratch copy of the forecast, so the analysis
                                     itself is unaffected; one host synchronisation), and the
@@ -127,8 +130,8 @@ extern "C" {
                                 candidate in the multiply-add loop                         */
 #define LETKF_GRAM_TENSOR 3  /* (reported only) tensor cores: the Gram matrices of all grid points as
                                 one product over the observation points, three BF16 parts per
-                                operand (24 significant bits), FP32 sums; LETKF_MIXED's
-                                split-FP16 form on grids below 1,024 points                 */
+                                operand (24 significant bits), FP32 sums; and LETKF_MIXED's
+                                split-FP16 form                                             */
 
 /* ---- problem statement --------------------------------------------------
  * Follows the paper's statement of the problem (Sec. II-B): the grid, the
@@ -175,8 +178,8 @@ typedef struct letkf_stats {
     int32_t max_local_obs;     /* l_max: most observation points local to one point     */
     double  mean_local_obs;    /* average observation points per grid point             */
     int32_t n_chunks;          /* Gram/eigensolve launch pairs per analysis             */
-    int32_t eig_schedule;      /* LETKF_EIG_FUSED / SPLIT / SPLIT_CHECK in use; AUTO (0)
-                                  until the first analysis resolves it                   */
+    int32_t eig_schedule;      /* LETKF_EIG_* in use (see LETKF_EIG_AUTO for k > 64); AUTO
+                                  (0) until the first analysis resolves it               */
     int32_t cuda_error;        /* first cudaError_t that made a call of this handle
                                   return LETKF_ECUDA or LETKF_ENOMEM; 0 = none           */
     int32_t cycle_kernels;     /* kernel launches of the most recent letkf_cycle (or group

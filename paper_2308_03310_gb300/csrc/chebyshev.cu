@@ -97,12 +97,31 @@ double chebyshev_coefficients(double kappa, int n, double *ca, double *cb) {
 }
 
 // The approximations the schedule chooses from: for each kappa_max the smallest degree whose
-// error stays below 2e-8 (under FP32 rounding of the result), found once with
-// chebyshev_coefficients.  The sets beyond 16 serve k > kChebMaxK only and are built with it.
+// error stays below 2e-8 in FP64, found once with chebyshev_coefficients.  The kernel reads the
+// coefficients rounded to FP32; with them t^-1/2 and t^-1 are off by up to 6.9e-8 / 1.3e-7 at
+// kappa_max = 16, 8.4e-8 / 6.9e-7 at 80 and 2.7e-7 / 4.5e-6 at 400 (relative, at the far end of the
+// interval).  The sets beyond 16 serve k > kChebMaxK only and are built with it.  Against the split
+// eigensolve that served those points before, on the same A and c (k = 65, 100, 128; observation
+// errors falling across the grid, smooth and pointwise perturbations, innovations of noise and of a
+// truth drawn with the ensemble): mean increment off by 4.3e-8 to 1.9e-6 against 7.3e-7 to 2.4e-5,
+// the perturbations by 6.0e-8 to 9.5e-7 against 1.4e-6 to 1.1e-5; in every class of condition bounds
+// at most 0.65 (increment) and 0.28 times as far from the FP64 transform as the split schedule.
 // The sets 3.5, 5, 7, 12 and 14 save products where kappa is above 3: 250 x 187, k = 40 20.7 -> 19.0
 // a point (eigensolve phase 1.67 -> 1.56 ms), 256 x 256, k = 64 28.4 -> 28.1 (3.82 -> 3.76 ms), 192 x
 // 160, k = 128 13.4 -> 13.2.
 namespace {
+constexpr double kSetKappa[kChebBigSets] = {
+    1.0002, 1.005, 1.035, 1.1,  1.2,  1.35, 1.5, 1.75, 2.0, 2.5, 3.0, 3.5, 4.0, 5.0,
+    6.0,    7.0,   10.0,  12.0, 14.0, 16.0, 24,  36,   54,  80,  120, 180, 270, 400};
+constexpr int kSetDegree[kChebBigSets] = {1,  2,  3,  4,  5,  7,  8,  9,  10, 12,  13,  15,  16,  19,
+                                          21, 23, 28, 30, 33, 36, 44, 54, 67, 82, 100, 123, 151, 184};
+constexpr int set_coefs(int sets) {
+    int n = 0;
+    for (int s = 0; s < sets; ++s) n += kSetDegree[s] + 1;
+    return n;
+}
+static_assert(set_coefs(kChebBigSets) <= kChebCoefs, "the table holds every set's coefficients");
+
 void cheb_set(ChebTable &t, int s, double kmax, int n) {
     // the interval the kernel maps onto [-1, 1] is the FP32 kappa_max: the coefficients and the
     // degree are those of that interval
@@ -121,20 +140,12 @@ const ChebTable &cheb_table(int k) {
     static ChebTable t, big;
     static std::once_flag once, once_big;
     std::call_once(once, [] {
-        const double kmax[kChebSets] = {1.0002, 1.005, 1.035, 1.1, 1.2, 1.35, 1.5,
-                                        1.75,   2.0,   2.5,   3.0, 3.5, 4.0,  5.0,
-                                        6.0,    7.0,   10.0,  12.0, 14.0, 16.0};
-        const int deg[kChebSets] = {1,  2,  3,  4,  5,  7,  8,  9,  10, 12,
-                                    13, 15, 16, 19, 21, 23, 28, 30, 33, 36};
-        for (int s = 0; s < kChebSets; ++s) cheb_set(t, s, kmax[s], deg[s]);
+        for (int s = 0; s < kChebSets; ++s) cheb_set(t, s, kSetKappa[s], kSetDegree[s]);
     });
     if (k <= kChebMaxK) return t;
     std::call_once(once_big, [] {
         big = t;
-        const double kmax[kChebBigSets - kChebSets] = {24, 36, 54, 80, 120, 180, 270, 400};
-        const int deg[kChebBigSets - kChebSets] = {44, 54, 67, 82, 100, 123, 151, 184};
-        for (int i = 0; i < kChebBigSets - kChebSets; ++i)
-            cheb_set(big, kChebSets + i, kmax[i], deg[i]);
+        for (int s = kChebSets; s < kChebBigSets; ++s) cheb_set(big, s, kSetKappa[s], kSetDegree[s]);
     });
     return big;
 }
@@ -146,7 +157,10 @@ const ChebTable &cheb_table(int k) {
 // the same points take the same schedule, although products have become cheaper (break-even
 // measured since at 7, 17, 24, 28, 31 and 55 for k = 8, 16, 20, 24, 32 and 40 to 64; a point beyond
 // goes to the rational schedule).  k > 64: the alternative is the split eigensolve, ~2.5 us a
-// point at k = 128 against ~10 ns a product: every set is used up to degree 1.4 k.
+// point at k = 128 against ~10 ns a product: every set is used up to degree 7k/5 + 5, that is
+// up to kappa 80 (degree 82) at k = 65, 180 (123) at k = 100 and 400 (184) at k = 128.  Where
+// every point is beyond, the transform's look at the bounds costs 2 % of the phase at k = 72 (4.38
+// -> 4.48 ms at 64 x 64), 0.4 % at k = 128.
 int cheb_max_set(int k) {
     const ChebTable &t = cheb_table(k);
     const int nsets = k <= kChebMaxK ? kChebSets : kChebBigSets;

@@ -207,7 +207,7 @@ cudaError_t launch_eigen_rational(const EigArgs &a, const EigSplit &sp, int grid
 // condition bound is used.
 constexpr int kChebSets = 20;
 constexpr int kChebMaxK = 64;       // LETKF_EIG_CHEBYSHEV; beyond, up to kChebSplitMaxK, AUTO may
-constexpr int kChebSplitMaxK = 128;  // choose it, with the sets up to kappa 400
+constexpr int kChebSplitMaxK = 128;  // choose it (kappa to 80 at k = 65, 180 at 100, 400 at 128)
 constexpr int kChebBigSets = 28;
 constexpr int kChebCoefs = 1136;
 struct ChebTable {
