@@ -469,7 +469,10 @@ int enqueue_obs(letkf_handle *h) {
     o.yf = h->yf;
     o.yb = h->yb;
     o.ybar = h->ybar;
-    if (h->gemm) o.clear = h->status + kGemmFlag;
+    if (h->gemm) {
+        o.clear = h->status + kGemmFlag;
+        o.clear_rows = h->zbad;
+    }
     CK(lk::launch_obs_operator(o, h->stream));
     return LETKF_OK;
 }

@@ -629,6 +629,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegSum));
         const int half = (warp - kWarpSum) >> 2;   // columns (grid points) 128 half ..
         const uint32_t src = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + half * (kPts / 2);
+        const int flagged = *a.flag;               // written before this launch
         uint32_t g = 0;
         bool ok = true;
         for (int it = blockIdx.x; it < nitems && !abort_flag && ok; it += gridDim.x) {
@@ -682,7 +683,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
         if (!ok) fail();
-        else if (*a.flag)   // written before this launch; the lanes' own stores are the operands
+        else if (flagged)   // the lanes' own stores are the operands
             for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
                 int tx0, ty0;
                 const int mt = item_at(it, tx0, ty0);
@@ -701,7 +702,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // z of every observation point in bin order, three BF16 parts: block per observation point, two
 // neighbouring pairs per thread and round.  pairs[m] = i | j << 16 (j = k: the innovation), -1:
-// padding.  An entry that is not finite becomes zero; its row is marked in zbad, and the flag raised.
+// padding.  An entry that is not finite becomes zero; its row is marked in zbad, and the flag raised
+// (both cleared by the observation operator).
 __global__ void __launch_bounds__(256) gram_z_kernel(const __grid_constant__ GemmArgs a) {
     __shared__ float dy[3][132];
     __shared__ float ri[3];
@@ -739,10 +741,9 @@ __global__ void __launch_bounds__(256) gram_z_kernel(const __grid_constant__ Gem
         *reinterpret_cast<__nv_bfloat162 *>(a.z + part + at) = mb;
         *reinterpret_cast<__nv_bfloat162 *>(a.z + 2 * part + at) = lb;
     }
-    const int any = __syncthreads_or(bad);
-    if (threadIdx.x == 0) {
-        a.zbad[j] = any;
-        if (any) atomicOr(a.flag, 1);
+    if (bad) {
+        a.zbad[j] = 1;
+        atomicOr(a.flag, 1);
     }
 }
 

@@ -53,7 +53,7 @@ struct ObsOpArgs {
     float *yf;              // [nmem][L*V] h(x_m)
     float *yb;              // [L*V][kp]  h(x_m) - mean, zero in columns k..kp-1
     float *ybar;            // [L*V]      mean minus the variable's reference (1 for rho)
-    int *clear = nullptr;   // a device word set to zero (optional)
+    int *clear = nullptr, *clear_rows = nullptr;   // a device word, and L words, set to zero (optional)
 };
 cudaError_t launch_obs_operator(const ObsOpArgs &a, cudaStream_t s);
 cudaError_t launch_count_local(const ObsNet &net, int nx, int ny, int *nloc, cudaStream_t s);

@@ -23,6 +23,7 @@ __global__ void __launch_bounds__(128) obs_operator_kernel(ObsOpArgs a) {
     for (int l = warp; l < a.L; l += nwarps) {
         const int2 o = a.xy[l];
         const size_t p = (size_t)o.y * a.nx + o.x;
+        if (a.clear_rows && lane == 0) a.clear_rows[l] = 0;
         float val[5][3];
         float sum[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
