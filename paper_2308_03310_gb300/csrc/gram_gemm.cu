@@ -629,7 +629,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegSum));
         const int half = (warp - kWarpSum) >> 2;   // columns (grid points) 128 half ..
         const uint32_t src = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + half * (kPts / 2);
-        const int flagged = *a.flag;               // written before this launch
         uint32_t g = 0;
         bool ok = true;
         for (int it = blockIdx.x; it < nitems && !abort_flag && ok; it += gridDim.x) {
@@ -683,7 +682,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
         if (!ok) fail();
-        else if (flagged)   // the lanes' own stores are the operands
+        else if (*a.flag)   // written before this launch (read here: a register held through the
+                            // sums, or a shared word, costs 2 % of the kernel)
             for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
                 int tx0, ty0;
                 const int mt = item_at(it, tx0, ty0);
@@ -725,13 +725,16 @@ __global__ void __launch_bounds__(256) gram_z_kernel(const __grid_constant__ Gem
             if (p >= 0)
                 z_entry(V, [&](int v) { return make_float3(dy[v][p & 0xffff], dy[v][p >> 16], ri[v]); },
                         hi[h], lo[h]);
-            if (!z_finite(hi[h])) {
-                bad = true;
-                hi[h] = lo[h] = 0.0f;
-            }
         }
-        const __nv_bfloat162 hb = __floats2bfloat162_rn(hi[0], hi[1]);
-        const float2 hf = bf2f(hb);
+        __nv_bfloat162 hb = __floats2bfloat162_rn(hi[0], hi[1]);
+        float2 hf = bf2f(hb);
+        if (!isfinite(hf.x) || !isfinite(hf.y)) {   // (z_finite)
+            bad = true;
+            if (!isfinite(hf.x)) hi[0] = lo[0] = 0.0f;
+            if (!isfinite(hf.y)) hi[1] = lo[1] = 0.0f;
+            hb = __floats2bfloat162_rn(hi[0], hi[1]);
+            hf = bf2f(hb);
+        }
         const float a0 = (hi[0] - hf.x) + lo[0], a1 = (hi[1] - hf.y) + lo[1];
         const __nv_bfloat162 mb = __floats2bfloat162_rn(a0, a1);
         const float2 mf = bf2f(mb);
